@@ -1,5 +1,6 @@
 // extern "C" entry points of libuvc: argument checks, lamp conversion, and
 // dispatch to the kernels.  See include/uvc.h for the contract of each call.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -52,10 +53,17 @@ int lamp_to_device(const uvc_lamp* lamp, LampDev* out, float coord_bound, int64_
         out->oz[m] = lamp->offsets[m][2];
         out->pw[m] = w * lamp->power;   // source power w_m P (one FP32 rounding)
     }
+    out->zmin = out->zmax = out->oz[0];
+    for (int m = 1; m < lamp->K; ++m) {
+        out->zmin = std::min(out->zmin, out->oz[m]);
+        out->zmax = std::max(out->zmax, out->oz[m]);
+    }
+    const bool merged = g_wedge.load(std::memory_order_relaxed) != 0;
+    out->plates = merged ? 1 : 0;
     bool vertical = lamp->K >= 2 && lamp->K <= kWedgeMaxK;
     for (int m = 0; m < lamp->K && vertical; ++m) vertical = out->ox[m] == 0.f && out->oy[m] == 0.f;
     // the wedge search queues leaf indices in 27 bits (larger scenes search source by source)
-    out->wedge = vertical && max_tris <= kWedgeMaxTris && g_wedge.load(std::memory_order_relaxed) ? 1 : 0;
+    out->wedge = vertical && max_tris <= kWedgeMaxTris && merged ? 1 : 0;
     if (out->wedge) {
         const int K = lamp->K;
         const double z0 = out->oz[0], dz = ((double)out->oz[K - 1] - z0) / (K - 1);

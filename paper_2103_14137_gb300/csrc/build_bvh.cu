@@ -567,6 +567,7 @@ __device__ __forceinline__ float box_half_area(const float* lo, const float* hi)
 
 __global__ void k_collapse_level(const Node* __restrict__ nodes, const int* __restrict__ fin,
                                  const int* __restrict__ nin, int* __restrict__ fout, int* __restrict__ nout,
+                                 const int* __restrict__ leaf_loose, const int* __restrict__ node_loose,
                                  Node4* __restrict__ nodes4) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= *nin) return;
@@ -612,12 +613,13 @@ __global__ void k_collapse_level(const Node* __restrict__ nodes, const int* __re
         for (int a = 0; a < 3; ++a)
             o.q[3 * h + a] = make_float4(lo[2 * h][a], lo[2 * h + 1][a], hi[2 * h][a], hi[2 * h + 1][a]);
     o.r = make_int4(ref[0], ref[1], ref[2], ref[3]);
-    int leafmask = 0, innermask = 0, ninner = 0;
+    int leafmask = 0, innermask = 0, ninner = 0, loose = 0;
     for (int c = 0; c < 4; ++c) {
         if (ref[c] < 0) leafmask |= 1 << c;
         else if (ref[c] != kEmptyChild) { innermask |= 1 << c; ++ninner; }
+        if (ref[c] != kEmptyChild && (ref[c] < 0 ? leaf_loose[~ref[c]] : node_loose[ref[c]])) loose |= 1 << c;
     }
-    o.m = make_int4(leafmask, innermask, 0, 0);
+    o.m = make_int4(leafmask, innermask, loose, 0);
     nodes4[i] = o;
     if (ninner) {
         int at = atomicAdd(nout, ninner);
@@ -935,6 +937,7 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
                    align256(sizeof(Node4) * (size_t)ni) +
                    align256(sizeof(uint64_t) * (size_t)n) + align256(sizeof(int32_t) * (size_t)n) +
                    2 * align256(sizeof(float4) * (size_t)np) + align256(sizeof(int2) * (size_t)np) +
+                   align256(sizeof(float4) * 2 * kMaxPlates + sizeof(uint32_t) * (size_t)((np + 31) / 32)) +
                    align256(sizeof(float)) + align256(sizeof(int)) + 256;
     if (cudaMallocAsync(&sc->block, bytes, stream) != cudaSuccess) {
         cudaGetLastError();
@@ -950,10 +953,13 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
     sc->patch_s = pc.take<float4>(np);
     sc->patch_n = pc.take<float4>(np);
     sc->patch_excl = pc.take<int2>(np);
+    sc->plates = pc.take<float4>(2 * kMaxPlates);
+    pc.off += sizeof(uint32_t) * (size_t)((np + 31) / 32);   // the patch flags follow the plates
     sc->area_total = pc.take<float>(1);
     sc->status = pc.take<int>(1);
 
     // temporaries
+    const bool plates = !(flags_in & UVC_BUILD_LBVH_ONLY) && n > 1 && nt <= kPlateMaxTris;
     const int ntiles = (n + kSortTile - 1) / kSortTile;
     size_t tbytes = 3 * align256(sizeof(float4) * (size_t)n) +            // tri_lo, tri_hi, ref
                     align256(sizeof(uint64_t) * (size_t)n) +                // keys alt
@@ -966,7 +972,9 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
                     3 * align256(sizeof(int) * (size_t)ni) +                 // height, flags, depth
                     align256(sizeof(float) * (size_t)ni) +                   // subtree cost
                     align256(sizeof(int) * (size_t)n) +                      // leaf parents at pass start
-                    align256(sizeof(unsigned int) * 12) + align256(sizeof(int) * 2) +
+                    align256(sizeof(unsigned int) * 12) + align256(sizeof(int) * 4) +
+                    align256(sizeof(int) * (size_t)n) + align256(sizeof(int) * (size_t)ni) +   // loose leaves, nodes
+                    (plates ? align256(plates_work_bytes(nt)) : 0) +
                     align256(sizeof(int) * ((size_t)n + 2)) + 256;                    // collapse level counters
     void* tblock = nullptr;
     if (cudaMallocAsync(&tblock, tbytes, stream) != cudaSuccess) {
@@ -997,14 +1005,17 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
     float* cost = tc.take<float>(ni);
     int* leaf_parent0 = tc.take<int>(n);
     unsigned int* bounds = tc.take<unsigned int>(12);   // reference points lo/hi, triangle boxes lo/hi
-    int* errdepth = tc.take<int>(2);   // [0] = error bits, [1] = depth
+    int* errdepth = tc.take<int>(4);   // [0] = error bits, [1] = depth, [2] = plates, [3] = loose triangles
+    int* leaf_loose = tc.take<int>(n);
+    int* node_loose = tc.take<int>(ni);
+    char* plates_work = plates ? tc.take<char>(plates_work_bytes(nt)) : nullptr;
     int* level_counts = tc.take<int>((size_t)n + 2);   // four-wide nodes per level of the collapse
 
     cudaError_t e = cudaSuccess;
     unsigned int init_bounds[12] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u,
                                     0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
     e = cudaMemcpyAsync(bounds, init_bounds, sizeof(init_bounds), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(errdepth, 0, 2 * sizeof(int), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(errdepth, 0, 4 * sizeof(int), stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(sc->status, 0, sizeof(int), stream);
     if (e == cudaSuccess && ni) e = cudaMemsetAsync(flags, 0, sizeof(int) * (size_t)ni, stream);
     const int B = 256;
@@ -1043,6 +1054,10 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
                     k_restructure<<<(n + 127) / 128, 128, 0, stream>>>(n, T, leaf_parent0, flags);
                 }
             }
+            if (plates) {
+                cudaMemsetAsync(node_loose, 0, sizeof(int) * (size_t)ni, stream);
+                find_plates(sc, parent_leaf, parent_int, leaf_loose, node_loose, errdepth + 2, plates_work, stream);
+            }
             cudaMemsetAsync(errdepth + 1, 0, sizeof(int), stream);
             k_pack_nodes<<<(ni + B - 1) / B, B, 0, stream>>>(n, children, parent_int, leaf_lo, leaf_hi, node_lo,
                                                              node_hi, sc->nodes);
@@ -1055,7 +1070,7 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
     // one synchronisation: validation result, tree depth and the scene diameter
     // (clearance margin, traversal cut tolerance) come back to the host
     unsigned int host_bounds[12];
-    int host_ed[2] = {0, 0};
+    int host_ed[4] = {0, 0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_bounds, bounds, sizeof(host_bounds), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_ed, errdepth, sizeof(host_ed), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -1071,6 +1086,11 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
     if (host_ed[0] != 0) return fail(UVC_E_INVAL);
     sc->depth = host_ed[1];
     sc->depth4 = (sc->depth + 1) / 2;
+    if (plates && host_ed[2] <= kMaxPlates) {
+        sc->nplate = host_ed[2];
+        sc->nloose = host_ed[3];
+    }
+    if (!plates && ni) cudaMemsetAsync(leaf_loose, 0, (char*)(node_loose + ni) - (char*)leaf_loose, stream);
     if (n > 1 && !(flags_in & UVC_BUILD_LBVH_ONLY)) {
         // the greedy collapse, one launch per level of four-wide nodes; a path
         // of the four-wide tree advances at least one binary level per node,
@@ -1085,7 +1105,7 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
             const int64_t bound = L < 15 ? std::min<int64_t>(ni, int64_t(1) << (2 * L)) : ni;
             k_collapse_level<<<(int)((bound + B - 1) / B), B, 0, stream>>>(sc->nodes, L & 1 ? fb : fa, counters + L,
                                                                          L & 1 ? fa : fb, counters + L + 1,
-                                                                         sc->nodes4);
+                                                                         leaf_loose, node_loose, sc->nodes4);
         }
         if (cudaGetLastError() != cudaSuccess) return fail(UVC_E_CUDA);
     }

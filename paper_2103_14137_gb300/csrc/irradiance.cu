@@ -54,9 +54,13 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS) k_irradiance(Sce
     const int njb = (S.np + 31) >> 5;
     const int nchunk = (nc + kCandPerTask - 1) / kCandPerTask;
     const int64_t ntask = (int64_t)nchunk * njb;
-    for (int64_t task = (int64_t)blockIdx.x * kWarpsPerBlock + warp; task < ntask;
-         task += (int64_t)gridDim.x * kWarpsPerBlock) {
-        const int jb = (int)(task / nchunk), ic = (int)(task % nchunk);
+    // task = jb nchunk + ic, advanced by a fixed stride: one division each per
+    // warp, not per task
+    const int64_t stride = (int64_t)gridDim.x * kWarpsPerBlock;
+    const int djb = (int)(stride / nchunk), dic = (int)(stride % nchunk);
+    int64_t task = (int64_t)blockIdx.x * kWarpsPerBlock + warp;
+    int jb = (int)(task / nchunk), ic = (int)(task % nchunk);
+    for (; task < ntask; task += stride) {
         const int j = jb * 32 + lane;
         const PatchLane P = load_patch(S, j);
         int cache = -1;
@@ -66,6 +70,12 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS) k_irradiance(Sce
                 WEDGE ? irradiance_wedge<COUNT>(S, cand, nc, L, i, jb, lane, stack, ws, vis, njb, P, cache, ctr)
                       : irradiance_entry<COUNT>(S, cand, nc, L, i, jb, lane, stack, vis, njb, P, cache, ctr);
             if (P.valid) A[(size_t)i * lda + j] = E;
+        }
+        jb += djb;
+        ic += dic;
+        if (ic >= nchunk) {
+            ic -= nchunk;
+            ++jb;
         }
     }
 }

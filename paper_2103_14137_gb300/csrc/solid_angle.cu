@@ -124,7 +124,7 @@ __device__ __forceinline__ uint32_t packet_to(const SceneView& S, float ox, floa
     uint32_t failed;
     int hit_tri = -1;
     const uint32_t occl =
-        cached_mask | warp_occluded<false>(S, r, want & ~cached_mask, stack, lane, failed, nullptr, hit_tri);
+        cached_mask | warp_occluded<false>(S, r, want & ~cached_mask, ~0u, stack, lane, failed, nullptr, hit_tri);
     if (hit_tri >= 0) cache = hit_tri;
     failed_all |= failed;
     return occl;
@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
         const int j = jb * 32 + lane;
         const PatchLane P = load_patch(S, j);
         const float* g = ptri + 18 * (size_t)(P.valid ? j : 0);
+        const bool flagged = WEDGE && S.nplate != 0 && plate_flag(S, jb, lane);
         const int tmask = used_triangles(g, P.valid);
         const float inv_area = P.valid && P.s.w > 0.f ? __frcp_rn(__fmul_rn(kFourPi, P.s.w)) : 0.f;
         int cache = -1;
@@ -179,13 +180,13 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
                         dq = 0.f;
                         gxq = 0.f;
                         gyq = 0.f;
-                        if (want_q) wedge_setup_point(L, cx, cy, cz, pq, want_q, lane, ws, dq, gxq, gyq);
+                        if (want_q) wedge_setup_point(L, cx, cy, cz, pq, want_q, dq, gxq, gyq);
                         szq = pq.z;
                         lq = 1.f;
                     }
                     uint32_t fq;
                     const uint32_t oc = wedge_search<false>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex,
-                                                            lane, stack, ws, cache, fq, nullptr);
+                                                            flagged, lane, stack, ws, cache, fq, nullptr);
                     failed_all |= fq;
                     if (q < 0) {
                         vis_c = ((fq >> lane) & 1u) ? 0u : (facing & ~oc);
@@ -240,7 +241,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
                 uint32_t failed;
                 int hit_tri = -1;
                 const uint32_t occl = cached_mask | warp_occluded<false>(S, r, facing_mask & ~cached_mask & ~settled_mask,
-                                                                         stack, lane, failed, nullptr, hit_tri);
+                                                                         ~0u, stack, lane, failed, nullptr, hit_tri);
                 if (hit_tri >= 0) cache = hit_tri;
                 failed_all |= failed;
                 const uint32_t visible = facing_mask & ~occl & ~failed;

@@ -29,7 +29,8 @@ struct __align__(16) Node {
 //   r = child refs: >= 0 four-wide node (indexed like the binary node it came
 //       from), < 0 leaf ~k, kEmptyChild for an unused slot (its box is a point
 //       far outside the scene, so no segment enters it)
-//   m = (bit c set: child c is a leaf, bit c set: child c is a four-wide node, 0, 0)
+//   m = (bit c set: child c is a leaf, bit c set: child c is a four-wide node,
+//        bit c set: child c holds a triangle that lies in no plate, 0)
 constexpr int kEmptyChild = 0x7fffffff;
 struct __align__(16) Node4 {
     float4 q[6];
@@ -43,17 +44,27 @@ struct __align__(16) Node4 {
 constexpr int kWedgeMaxK = 16;
 constexpr int64_t kWedgeMaxTris = int64_t(1) << 27;
 
+// Plates (plates.cu): flat axis-aligned rectangles tiled by the mesh's
+// triangles.  The searches test a room's plates 32 at a time, one per lane,
+// before the hierarchy; past kMaxPlates that would cost more than it saves.
+constexpr int kMaxPlates = 1024;
+constexpr int64_t kPlateMaxTris = int64_t(1) << 27;   // edge numbers are 4 k + e in 32 bits
+
 // Lamp as seen by the kernels: source offsets and source powers w_m * P.
 // wedge = 1: every offset is vertical (x = y = 0), 2 <= K <= kWedgeMaxK, and
 // the wedge traversal is switched on (uvc_set_wedge_traversal).
 // Wedge lamps whose offsets rise evenly (off_m.z within 1/64 of a step of
 // wz0 + m dz, dz > 0) have wuniform = 1 and wz0, wrdz = 1/dz set: the
 // sources in a height interval are then a range of indices.
+// plates = 1: the searches for this lamp may decide segments at the scene's
+// plates (the setting of uvc_set_wedge_traversal).  zmin, zmax: the extreme
+// offsets in z.
 struct LampDev {
     int K;
-    int wedge;
+    int16_t wedge, plates;
     int wuniform;
     float wz0, wrdz;
+    float zmin, zmax;
     float ox[UVC_MAX_SOURCES], oy[UVC_MAX_SOURCES], oz[UVC_MAX_SOURCES];
     float pw[UVC_MAX_SOURCES];
 };
@@ -84,6 +95,9 @@ struct uvc_scene {
     float4* patch_n = nullptr;    // [np] (normal, clearance): see k_clearance
     int2* patch_excl = nullptr;   // [np]
     float* area_total = nullptr;  // [1]
+    float4* plates = nullptr;     // [kMaxPlates][2]: (lo, axis bits), (hi, 0); then one flag bit per patch
+    int32_t nplate = 0;
+    int32_t nloose = 0;           // triangles of no plate
     int* status = nullptr;        // [1] device status word (0 = ok)
     cudaStream_t build_stream = nullptr;
     // lowered traversal limits (uvc_scene_set_limits); 0 = the built-in bound
@@ -102,6 +116,11 @@ int status_from_cuda(cudaError_t e);
 // BVH build (build_bvh.cu)
 int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt, const uvc_patches* patches,
                 int64_t np, uint32_t flags, cudaStream_t stream, uvc_scene** out);
+
+// plates (plates.cu)
+size_t plates_work_bytes(int64_t nt);
+void find_plates(uvc_scene* sc, const int* parent_leaf, const int* parent_int, int* leaf_loose, int* node_loose,
+                 int* counts, void* work, cudaStream_t stream);
 
 // irradiance (irradiance.cu)
 int irradiance_matrix(const uvc_scene* sc, const float* cand, int64_t nc, const LampDev& lamp, float* A,
