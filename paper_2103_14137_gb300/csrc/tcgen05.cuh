@@ -61,10 +61,13 @@ __device__ __forceinline__ void dealloc(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// Shared-memory matrix descriptor, K-major without swizzle: 8-row x 16-byte
-// core matrices, `lbo` bytes between the two core matrices of an 8-row group
-// along K, `sbo` bytes between consecutive 8-row groups; descriptor version 1
-// (bits 46-47), no swizzle (bits 61-63 = 0).
+// Shared-memory matrix descriptor without swizzle: 8-row x 16-byte core
+// matrices.  K-major operands (a row holds 16 bytes along K): `lbo` bytes
+// between the two core matrices of an 8-row group along K, `sbo` bytes between
+// consecutive 8-row groups.  MN-major operands (a row holds 16 bytes along M
+// or N, the 8 rows go along K): `sbo` bytes between core matrices along M or
+// N, `lbo` bytes between those along K.  Descriptor version 1 (bits 46-47), no
+// swizzle (bits 61-63 = 0).
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
     return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
@@ -72,11 +75,12 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
 
 // Instruction descriptor of .kind::f16 / .kind::tf32 with an FP32 accumulator:
 // D format bits 4-5 (1 = F32), A and B formats bits 7-9 and 10-12 (kind::f16:
-// 0 = F16, 1 = BF16; kind::tf32: 2 = TF32; A and B the same), both operands
-// K-major (bits 15, 16 = 0), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
+// 0 = F16, 1 = BF16; kind::tf32: 2 = TF32; A and B the same), bits 15 and 16
+// set where A and B are MN-major, N >> 3 in bits 17-22, M >> 4 in bits 24-28.
 constexpr uint32_t kFmtBF16 = 1, kFmtTF32 = 2;
-constexpr uint32_t idesc_f32acc(uint32_t fmt, int M, int N) {
-    return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+__host__ __device__ constexpr uint32_t idesc_f32acc(uint32_t fmt, int M, int N, bool a_mn = false, bool b_mn = false) {
+    return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 // D (tensor memory) = A B (+ D when `accumulate`), issued by one thread.
