@@ -38,7 +38,7 @@ std::atomic<int> g_wedge{1};
 // 0 = CUDA cores (defined in fluence.cu)
 extern std::atomic<int> g_fluence_tc;
 
-int lamp_to_device(const uvc_lamp* lamp, LampDev* out, float coord_bound, int64_t max_tris) {
+int lamp_to_device(const uvc_lamp* lamp, LampDev* out, float coord_bound, int64_t max_tris, bool per_4pi) {
     if (!lamp || lamp->K < 1 || lamp->K > UVC_MAX_SOURCES) return UVC_E_INVAL;
     if (!std::isfinite(lamp->power) || lamp->power < 0.f) return UVC_E_INVAL;
     std::memset(out, 0, sizeof(*out));
@@ -51,7 +51,7 @@ int lamp_to_device(const uvc_lamp* lamp, LampDev* out, float coord_bound, int64_
         out->ox[m] = lamp->offsets[m][0];
         out->oy[m] = lamp->offsets[m][1];
         out->oz[m] = lamp->offsets[m][2];
-        out->pw[m] = w * lamp->power;   // source power w_m P (one FP32 rounding)
+        out->pw[m] = per_4pi ? (float)((double)w * (double)lamp->power / (4.0 * M_PI)) : w * lamp->power;
     }
     out->zmin = out->zmax = out->oz[0];
     for (int m = 1; m < lamp->K; ++m) {
@@ -171,7 +171,7 @@ int uvc_irradiance_raster(const uvc_scene* scene, const float* tri_normal, const
                           uvc_stream_t stream) {
     if (!scene || !uvc::count_ok(nc) || nc > INT32_MAX || R < 1 || R > 4096) return UVC_E_INVAL;
     uvc::LampDev L;
-    int rc = uvc::lamp_to_device(lamp, &L, scene->coord_bound, scene->nt);
+    int rc = uvc::lamp_to_device(lamp, &L, scene->coord_bound, scene->nt, false);
     if (rc != UVC_OK) return rc;
     if (lda < scene->nt) return UVC_E_INVAL;
     if (nc > 0 && scene->nt > 0 && (!cand || !A || !tri_normal || !workspace)) return UVC_E_INVAL;

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
         const float* g = ptri + 18 * (size_t)(P.valid ? j : 0);
         const bool flagged = WEDGE && S.nplate != 0 && plate_flag(S, jb, lane);
         const int tmask = used_triangles(g, P.valid);
-        const float inv_area = P.valid && P.s.w > 0.f ? __frcp_rn(__fmul_rn(kFourPi, P.s.w)) : 0.f;
+        const float inv_area = P.valid && P.s.w > 0.f ? __frcp_rn(P.s.w) : 0.f;
         int cache = -1;
         const int i1 = min(nc, (ic + 1) * kAreaCandPerTask);
         for (int i = ic * kAreaCandPerTask; i < i1; ++i) {
@@ -165,8 +165,8 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
             uint32_t failed_all = 0;
             if (WEDGE) {
                 uint32_t want;
-                float lend, dmax, gx, gy;
-                const uint32_t facing = wedge_setup_patch(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy);
+                float lend, dmax, gx, gy, sum;
+                const uint32_t facing = wedge_setup_patch(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, sum);
                 uint32_t vis_c = 0u, all = 0u;   // all: sources that saw every check point so far
                 // q = -1: the centroid; q = 0..5: the check points.  One call site of
                 // the (large, inlined) wedge search keeps the kernel's code small.
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
                     E = __fadd_rn(E, __fmul_rn(__fmul_rn(L.pw[m], om), inv_area));
                     ++closed;
                 } else if (vis_c) {
-                    E = __fadd_rn(E, __fmul_rn(L.pw[m], __fdiv_rn(nv, __fmul_rn(__fmul_rn(kFourPi, d2), d))));
+                    E = __fadd_rn(E, source_term(L.pw[m], nv, d2));
                 }
             }
             if (P.valid) {

@@ -22,7 +22,6 @@ namespace {
 #endif
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr float kFourPi = 12.566370614359172f;
 // 1 + 2^-20: widening of the far slab distance; covers the relative rounding
 // of (b - o) * (1/d) (three roundings) with a wide margin.
 constexpr float kFarScale = 1.0f + 9.5367431640625e-07f;
@@ -320,6 +319,27 @@ __device__ uint32_t warp_occluded(const SceneView& S, const Ray& r, uint32_t ali
     return traverse4<COUNT>(S, r, alive, all, stack, lane, failed, ctr, hit_tri);
 }
 
+// Eq. (7) for one facing source: pw nv / d^3 from the squared distance d2.
+// d^-3 = r^3 (1 + 1.5 e) with r the approximate reciprocal square root of d2
+// (relative error 2^-22) and e = 1 - d2 r^2: the next term, 1.9 e^2, is below
+// 2^-43.  Five roundings, as with a rounded square root and division (and half
+// of the one of r^2, which e cancels in part), but no slow path to branch to
+// and half the instructions.  Distances whose cube leaves FP32 take the plain
+// form.
+constexpr float kTermMin = 1e-24f, kTermMax = 1e24f;
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float source_term(float pw, float nv, float d2) {
+    if (!(d2 >= kTermMin && d2 <= kTermMax)) return __fmul_rn(pw, __fdiv_rn(nv, __fmul_rn(d2, sqrtf(d2))));
+    const float r = rsqrt_approx(d2), r2 = __fmul_rn(r, r), r3 = __fmul_rn(r2, r);
+    const float f = __fmaf_rn(d2, r2, -1.f);
+    const float w = __fmaf_rn(__fmul_rn(f, -1.5f), r3, r3);
+    return __fmul_rn(pw, __fmul_rn(nv, w));
+}
+
 // One source's terms for the patch point s (normal n): v = o - s as the
 // rounded difference h plus its exact error (TwoSum), <n, v> with an
 // error-free dot product (TwoProduct + TwoSum) rounded once, and |h|^2.  Both
@@ -396,16 +416,17 @@ __device__ __forceinline__ PatchLane load_patch(const SceneView& S, int j) {
 //   clear     the wedge box test misses the rectangle's box (a search would
 //             enter no box inside it), or the segment stays well on one side
 //             of the plane, or crosses it well outside: none of them hits
-//   open      anything nearer to a border, an end or the plane's own
-//             direction; only these segments go on to the search
+//   open      anything nearer to a border or an end; only these segments go
+//             on to the search
 // so every visibility bit is the search's own.  "Well": the test's rounding
 // moves a triangle, seen along the segment, by about 2^-22 of the distances
 // involved (subtractions 2^-24, shear 2^-23); the margin is 8 times that, and
 // divided by the segment's cosine with the plane's normal within the plane.
-// Cosines below 1/64 stay open.  Off the plane 2^-14 of the distances is asked
-// for, as the rounding of a thin triangle's barycentric coordinates moves a
-// hit along it.  Both are taken of the scene's diagonal plus the longest
-// segment.  NaN and infinities fail the comparisons and stay open.
+// Off the plane 2^-14 of the distances is asked for: the rounding of a
+// triangle's barycentric coordinates (2^-22 times its 1 : 32 at most, over the
+// cosine) moves a hit by that part of its length along the segment, 2^-17 of
+// it along the normal.  Both are taken of the scene's diagonal plus the
+// longest segment.  NaN and infinities fail the comparisons and stay open.
 //
 // Which plates the packet's wedges can reach is found 32 at a time, a plate
 // per lane, against the packet's shaft: the hull's box, the two vertical
@@ -520,7 +541,7 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
                         const float ho = isx ? cx - lo.x : cy - lo.y, ga = isx ? gx : gy, ig = isx ? sl.igx : sl.igy;
                         const float gb = isx ? gy : gx, hs = ho + ga;
                         const float lb = isx ? lo.y - cy : lo.x - cx, ub = isx ? hi.y - cy : hi.x - cx;
-                        if (fminf(fabsf(ho), fabsf(hs)) >= far_off && fabsf(ga) * 64.f >= dmax) {
+                        if (fminf(fabsf(ho), fabsf(hs)) >= far_off) {
                             const float lam = -ho * ig, m = near_in * dmax * fabsf(ig);
                             const float t = fabsf(fmaf(lam, gb, -0.5f * (lb + ub))) - 0.5f * (ub - lb);
                             if (ho * hs > 0.f || t > m) {
@@ -542,7 +563,7 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
                         if (fabsf(hs) >= far_off)
                             for (int q = 0; q < K; ++q) {
                                 const float hm = zsrc(q) - lo.z, dz = hm - hs;
-                                if (fabsf(hm) >= far_off && fabsf(dz) * 64.f >= dmax) {
+                                if (fabsf(hm) >= far_off) {
                                     const float ig = rcp_approx(dz), lam = hm * ig, m = near_in * dmax * fabsf(ig);
                                     const float t = fmaxf(fabsf(fmaf(lam, gx, xc)) - hx, fabsf(fmaf(lam, gy, yc)) - hy);
                                     if (hm * hs > 0.f || t > m) clear |= 1u << q;
@@ -630,7 +651,7 @@ __device__ __forceinline__ float irradiance_entry(const SceneView& S, const floa
         if (vis && lane == 0) vis[((size_t)m * nc + i) * nwords + jb] = visible;
         if ((failed >> lane) & 1u) bad = true;
         if ((visible >> lane) & 1u) {
-            E = __fadd_rn(E, __fmul_rn(L.pw[m], __fdiv_rn(nv, __fmul_rn(__fmul_rn(kFourPi, d2), d))));
+            E = __fadd_rn(E, source_term(L.pw[m], nv, d2));
         }
     }
     return bad ? __int_as_float(0x7fffffff) : E;
@@ -1009,16 +1030,22 @@ __device__ __forceinline__ void wedge_traverse(const SceneView& S, const LampDev
     }
 }
 
-// Set-up of the segments from candidate c's sources to the lane's patch point
-// (the arithmetic of source_terms, source by source; what a vertical lamp's
-// sources share is computed once): their Eq. (7) terms go to shared memory;
-// returns the facing sources and, in `want`, those that need a search (facing,
-// longer than the clearance cut), with the largest cut parameter `lend`, the
-// longest such segment `dmax` and the common horizontal direction (gx, gy).
+// a - b, rounded once, for both halves (m1 = -1, -1).
+__device__ __forceinline__ float2 sub2(float2 a, float2 b, float2 m1) { return __ffma2_rn(b, m1, a); }
+
+// Set-up of the segments from candidate c's sources to the lane's patch point:
+// the arithmetic of source_terms and source_term, bit for bit, with what a
+// vertical lamp's sources share computed once and two sources at a time in
+// packed FP32x2 (one scalar source at a time took 2.9 ms of a 10.5 ms ward
+// matrix).  Their Eq. (7) terms (0 where the source does not face) go to
+// shared memory, and their sum in source order to `sum`.  Returns the facing
+// sources and, in `want`, those that need a search (facing, longer than the
+// clearance cut), with the largest cut parameter `lend`, the longest such
+// segment `dmax` and the common horizontal direction (gx, gy).
 __device__ __forceinline__ uint32_t wedge_setup_patch(const SceneView& S, const LampDev& L, float cx, float cy,
                                                       float cz, const PatchLane& P, int lane, const WedgeSmem& ws,
                                                       uint32_t& want, float& lend, float& dmax, float& gx,
-                                                      float& gy) {
+                                                      float& gy, float& sum) {
     const float4 s4 = P.s, n4 = P.n;
     const float hx = __fsub_rn(cx, s4.x), hy = __fsub_rn(cy, s4.y);
     const float qx = __fsub_rn(hx, cx), qy = __fsub_rn(hy, cy);
@@ -1036,37 +1063,63 @@ __device__ __forceinline__ uint32_t wedge_setup_patch(const SceneView& S, const 
         err0 = __fadd_rn(err0, __fadd_rn(q, e2));
         err0 = __fmaf_rn(n4.y, ly, err0);
     }
-    const float cut = __fmaf_rn(0.99f, P.n.w, -S.cut_eps);
+    const float2 m1 = make_float2(-1.f, -1.f), acc = make_float2(acc0, acc0), err = make_float2(err0, err0);
+    const float2 nz = make_float2(n4.z, n4.z), nzn = make_float2(-n4.z, -n4.z), sz = make_float2(s4.z, s4.z);
+    const float2 szn = make_float2(-s4.z, -s4.z), c2 = make_float2(cz, cz);
+    const float2 hx2 = make_float2(hx, hx), hy2 = make_float2(hy, hy);
     uint32_t facing = 0;
-    want = 0;
-    dmax = 0.f;
+    float far2 = 0.f;
+    sum = 0.f;
+    for (int m = 0; m < L.K; m += 2) {
+        const int k = min(m + 1, L.K - 1);   // an odd lamp's last source twice; its second half is dropped
+        const float2 oz = __fadd2_rn(c2, make_float2(L.oz[m], L.oz[k]));
+        const float2 hz = sub2(oz, sz, m1), qz = sub2(hz, oz, m1);
+        const float2 lz = __fadd2_rn(sub2(oz, sub2(hz, qz, m1), m1), sub2(szn, qz, m1));
+        const float2 pn = __fmul2_rn(nzn, hz), e3 = __ffma2_rn(nz, hz, pn);   // pn = -(n.z h.z)
+        const float2 s = sub2(acc, pn, m1), z = sub2(s, acc, m1);
+        const float2 q = sub2(sub2(acc, sub2(s, z, m1), m1), __fadd2_rn(pn, z), m1);
+        const float2 nv = __fadd2_rn(s, __ffma2_rn(nz, lz, __fadd2_rn(err, __fadd2_rn(q, e3))));
+        const float2 d2 = __ffma2_rn(hx2, hx2, __ffma2_rn(hy2, hy2, __fmul2_rn(hz, hz)));
+        const float2 r = make_float2(rsqrt_approx(d2.x), rsqrt_approx(d2.y));
+        const float2 r2 = __fmul2_rn(r, r), r3 = __fmul2_rn(r2, r), f = __ffma2_rn(d2, r2, m1);
+        const float2 w = __ffma2_rn(__fmul2_rn(f, make_float2(-1.5f, -1.5f)), r3, r3);
+        float2 t = __fmul2_rn(make_float2(L.pw[m], L.pw[k]), __fmul2_rn(nv, w));
+        bool f0 = nv.x > 0.f, f1 = nv.y > 0.f && k > m;
+        if (!(fminf(d2.x, d2.y) >= kTermMin && fmaxf(d2.x, d2.y) <= kTermMax)) {
+            f0 = f0 && d2.x > 0.f;
+            f1 = f1 && d2.y > 0.f;
+            t = make_float2(source_term(L.pw[m], nv.x, d2.x), source_term(L.pw[k], nv.y, d2.y));
+        }
+        t.x = f0 ? t.x : 0.f;
+        t.y = f1 ? t.y : 0.f;
+        ws.term[m * 32 + lane] = t.x;
+        if (k > m) ws.term[k * 32 + lane] = t.y;
+        sum = __fadd_rn(__fadd_rn(sum, t.x), t.y);
+        far2 = fmaxf(far2, fmaxf(f0 ? d2.x : 0.f, f1 ? d2.y : 0.f));
+        facing |= ((uint32_t)f0 << m) | ((uint32_t)f1 << k);
+    }
+    if (!P.valid) facing = 0u;
     gx = -hx;
     gy = -hy;
-    for (int m = 0; m < L.K; ++m) {
-        const float oz = __fadd_rn(cz, L.oz[m]);
-        const float hz = __fsub_rn(oz, s4.z), qz = __fsub_rn(hz, oz);
-        const float lz = __fadd_rn(__fsub_rn(oz, __fsub_rn(hz, qz)), __fsub_rn(-s4.z, qz));
-        const float p3 = __fmul_rn(n4.z, hz);
-        const float e3 = __fmaf_rn(n4.z, hz, -p3);
-        const float s = __fadd_rn(acc0, p3);
-        const float z = __fsub_rn(s, acc0);
-        const float q = __fadd_rn(__fsub_rn(acc0, __fsub_rn(s, z)), __fsub_rn(p3, z));
-        const float nv = __fadd_rn(s, __fmaf_rn(n4.z, lz, __fadd_rn(err0, __fadd_rn(q, e3))));
-        const float d2 = __fmaf_rn(hx, hx, __fmaf_rn(hy, hy, __fmul_rn(hz, hz)));
-        const float d = sqrtf(d2);
-        const bool fac = P.valid && nv > 0.f && d2 > 0.f;
-        ws.term[m * 32 + lane] = fac ? __fmul_rn(L.pw[m], __fdiv_rn(nv, __fmul_rn(__fmul_rn(kFourPi, d2), d))) : 0.f;
-        if (fac) {
-            facing |= 1u << m;
-            // a segment shorter than the cut meets no triangle at all
-            if (d > 1.001f * cut || 1.f - cut * __frcp_rn(d) > 0.f) {
-                want |= 1u << m;
-                dmax = fmaxf(dmax, d);
+    dmax = facing ? sqrtf(far2) : 0.f;
+    want = facing;
+    // a segment shorter than the cut meets no triangle at all; the lamp's
+    // distance tells most lanes that none of theirs is
+    const float cut = __fmaf_rn(0.99f, P.n.w, -S.cut_eps);
+    if (cut > 0.f && facing) {
+        const float dz = fmaxf(fmaxf(cz + L.zmin - s4.z, s4.z - (cz + L.zmax)), 0.f);
+        if (!(hx * hx + hy * hy + dz * dz > 1.003f * cut * cut)) {
+            dmax = 0.f;
+            for (uint32_t b = facing; b; b &= b - 1) {
+                const int m = __ffs(b) - 1;
+                const float hz = __fsub_rn(__fadd_rn(cz, L.oz[m]), s4.z);
+                const float d = sqrtf(__fmaf_rn(hx, hx, __fmaf_rn(hy, hy, __fmul_rn(hz, hz))));
+                if (1.f - cut * __frcp_rn(d) > 0.f) dmax = fmaxf(dmax, d);
+                else want &= ~(1u << m);
             }
         }
     }
-    lend = cut > 0.f ? 1.f - cut * __frcp_rn(dmax) : 1.f;   // rises with d: the longest segment's is the largest
-    if (!want) lend = 0.f;
+    lend = !want ? 0.f : (cut > 0.f ? 1.f - cut * __frcp_rn(dmax) : 1.f);   // rises with d: the longest segment's
     return facing;
 }
 
@@ -1218,24 +1271,28 @@ __device__ __forceinline__ float irradiance_wedge(const SceneView& S, const floa
                 cz = __ldg(&cand[3 * (size_t)i + 2]);
     uint32_t want;
     float lend, dmax, gx, gy;
-    const uint32_t facing = wedge_setup_patch(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy);
+    float E;
+    const uint32_t facing = wedge_setup_patch(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, E);
     uint32_t failed;
     const bool flagged = !COUNT && S.nplate != 0 && plate_flag(S, jb, lane);
     const uint32_t occl = wedge_search<COUNT>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, flagged, lane,
                                               stack, ws, cache, failed, ctr);
     const bool bad = (failed >> lane) & 1u;
     const uint32_t visible = bad ? 0u : (facing & ~occl);
-    float E = 0.f;
-    uint32_t word = 0u;   // lane m keeps source m's word (K <= 16), and the words leave in one store
-    for (int m = 0; m < L.K; ++m) {
-        const bool v = (visible >> m) & 1u;
-        if (vis) {
-            const uint32_t b = __ballot_sync(kFull, v);
-            if (lane == m) word = b;
-        }
-        if (v) E = __fadd_rn(E, ws.term[m * 32 + lane]);
+    if (!__all_sync(kFull, visible == facing)) {   // some source is hidden: the sum of the others
+        E = 0.f;
+        for (int m = 0; m < L.K; ++m)
+            if ((visible >> m) & 1u) E = __fadd_rn(E, ws.term[m * 32 + lane]);
     }
-    if (vis && lane < L.K) vis[((size_t)lane * nc + i) * nwords + jb] = word;
+    if (vis) {   // lane m keeps source m's word (K <= 16), and the words leave in one store
+        uint32_t word = __ballot_sync(kFull, P.valid);
+        if (!__all_sync(kFull, !P.valid || visible == (1u << L.K) - 1u))
+            for (int m = 0; m < L.K; ++m) {
+                const uint32_t b = __ballot_sync(kFull, (visible >> m) & 1u);
+                if (lane == m) word = b;
+            }
+        if (lane < L.K) vis[((size_t)lane * nc + i) * nwords + jb] = word;
+    }
     return bad ? __int_as_float(0x7fffffff) : E;
 }
 

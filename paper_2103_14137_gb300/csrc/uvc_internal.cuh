@@ -50,7 +50,8 @@ constexpr int64_t kWedgeMaxTris = int64_t(1) << 27;
 constexpr int kMaxPlates = 1024;
 constexpr int64_t kPlateMaxTris = int64_t(1) << 27;   // edge numbers are 4 k + e in 32 bits
 
-// Lamp as seen by the kernels: source offsets and source powers w_m * P.
+// Lamp as seen by the kernels: source offsets and source powers over the full
+// solid angle, w_m P / (4 pi) (rounded once; the rasteriser takes w_m P).
 // wedge = 1: every offset is vertical (x = y = 0), 2 <= K <= kWedgeMaxK, and
 // the wedge traversal is switched on (uvc_set_wedge_traversal).
 // Wedge lamps whose offsets rise evenly (off_m.z within 1/64 of a step of
@@ -72,7 +73,7 @@ struct LampDev {
 // Host: validate a lamp and convert it (api.cu); coord_bound is the largest
 // coordinate magnitude and max_tris the largest triangle count of the
 // scene(s) it will be used with.
-int lamp_to_device(const uvc_lamp* lamp, LampDev* out, float coord_bound, int64_t max_tris);
+int lamp_to_device(const uvc_lamp* lamp, LampDev* out, float coord_bound, int64_t max_tris, bool per_4pi = true);
 
 }  // namespace uvc
 
