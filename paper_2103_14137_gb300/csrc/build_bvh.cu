@@ -938,6 +938,7 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
                    align256(sizeof(uint64_t) * (size_t)n) + align256(sizeof(int32_t) * (size_t)n) +
                    2 * align256(sizeof(float4) * (size_t)np) + align256(sizeof(int2) * (size_t)np) +
                    align256(sizeof(float4) * 2 * kMaxPlates + sizeof(uint32_t) * (size_t)((np + 31) / 32)) +
+                   align256(sizeof(int2) * (size_t)n) +
                    align256(sizeof(float)) + align256(sizeof(int)) + 256;
     if (cudaMallocAsync(&sc->block, bytes, stream) != cudaSuccess) {
         cudaGetLastError();
@@ -955,6 +956,7 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
     sc->patch_excl = pc.take<int2>(np);
     sc->plates = pc.take<float4>(2 * kMaxPlates);
     pc.off += sizeof(uint32_t) * (size_t)((np + 31) / 32);   // the patch flags follow the plates
+    sc->tri_place = pc.take<int2>(n);
     sc->area_total = pc.take<float>(1);
     sc->status = pc.take<int>(1);
 

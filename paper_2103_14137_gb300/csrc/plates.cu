@@ -12,6 +12,8 @@
 // Then they cover the rectangle: added up as oriented areas, their boundary is
 // what the unshared edges leave, all of it on the border, so every point inside
 // is covered equally often, and at least once as no triangle has zero area.
+// Sets whose triangles' areas add up to more than the rectangle's (covered more
+// than once) are given up too: one triangle's place then holds no other.
 // Triangles thinner than 1 : 64 (twice the area against the longest edge
 // squared below 1/32) stay out: the searches' margins assume that the
 // intersection test's rounding moves a hit by far less than a triangle.
@@ -42,6 +44,8 @@ struct Flat {
     int ccw;
     float p;
     float u[3], v[3];
+    float longest;   // squared length of the longest edge
+    float area2;     // twice the area
 };
 
 __device__ __forceinline__ Flat flat_of(const float4* __restrict__ tri, int k) {
@@ -58,9 +62,10 @@ __device__ __forceinline__ Flat flat_of(const float4* __restrict__ tri, int k) {
     const float e1u = f.u[1] - f.u[0], e1v = f.v[1] - f.v[0], e2u = f.u[2] - f.u[0], e2v = f.v[2] - f.v[0];
     const float e3u = e2u - e1u, e3v = e2v - e1v;
     const float area2 = e1u * e2v - e1v * e2u;
-    const float longest = fmaxf(e1u * e1u + e1v * e1v, fmaxf(e2u * e2u + e2v * e2v, e3u * e3u + e3v * e3v));
-    if (!(fabsf(area2) * 32.f >= longest) || !(longest > 0.f)) f.axis = -1;
+    f.longest = fmaxf(e1u * e1u + e1v * e1v, fmaxf(e2u * e2u + e2v * e2v, e3u * e3u + e3v * e3v));
+    if (!(fabsf(area2) * 32.f >= f.longest) || !(f.longest > 0.f)) f.axis = -1;
     f.ccw = area2 > 0.f;
+    f.area2 = fabsf(area2);
     return f;
 }
 
@@ -172,12 +177,16 @@ __device__ __forceinline__ float unordered(unsigned u) {
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
-// Per set (at its root): bounding rectangle, triangle count, kStateBad.  The
+// Per set (at its root): bounding rectangle, triangle count, kStateBad, longest
+// edge (squared, as the bits of a positive float), twice the area (only looked
+// at to tell one covering from two).  The
 // triangles are in Morton order, so a warp holds few sets and adds each once.
 __global__ void k_plate_stats(const float4* __restrict__ tri, int nt, int* __restrict__ parent,
                               const unsigned* __restrict__ state, uint2* __restrict__ lo, uint2* __restrict__ hi,
-                              int2* __restrict__ cnt_bad) {
+                              int2* __restrict__ cnt_bad, unsigned* __restrict__ len, float* __restrict__ area2) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned edge = 0u;
+    float twice = 0.f;
     int root = -1;
     unsigned lu = ~0u, lv = ~0u, hu = 0u, hv = 0u;
     bool bad = false;
@@ -189,6 +198,8 @@ __global__ void k_plate_stats(const float4* __restrict__ tri, int nt, int* __res
         hu = ordered(fmaxf(f.u[0], fmaxf(f.u[1], f.u[2])));
         hv = ordered(fmaxf(f.v[0], fmaxf(f.v[1], f.v[2])));
         bad = (state[k] & kStateBad) != 0u;
+        edge = __float_as_uint(f.longest);
+        twice = f.area2;
     }
     unsigned todo = __ballot_sync(0xffffffffu, root >= 0);
     const int lane = threadIdx.x & 31;
@@ -199,12 +210,17 @@ __global__ void k_plate_stats(const float4* __restrict__ tri, int nt, int* __res
         const unsigned grp = __ballot_sync(0xffffffffu, in);
         const unsigned a = __reduce_min_sync(0xffffffffu, in ? lu : ~0u), b = __reduce_min_sync(0xffffffffu, in ? lv : ~0u);
         const unsigned c = __reduce_max_sync(0xffffffffu, in ? hu : 0u), d = __reduce_max_sync(0xffffffffu, in ? hv : 0u);
+        const unsigned l = __reduce_max_sync(0xffffffffu, in ? edge : 0u);
+        float sum = in ? twice : 0.f;
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         const bool any_bad = __any_sync(0xffffffffu, in && bad);
         if (lane == lead) {
             atomicMin(&lo[r].x, a);
             atomicMin(&lo[r].y, b);
             atomicMax(&hi[r].x, c);
             atomicMax(&hi[r].y, d);
+            atomicMax(&len[r], l);
+            atomicAdd(&area2[r], sum);
             atomicAdd(&cnt_bad[r].x, __popc(grp));
             if (any_bad) atomicOr(&cnt_bad[r].y, 1);
         }
@@ -237,12 +253,14 @@ __global__ void k_plate_check(const float4* __restrict__ tri, int nt, int* __res
 // kMaxPlates, and the scene then goes without.  plate_id: per root, or -1.
 __global__ void k_plate_select(const float4* __restrict__ tri, int nt, const int* __restrict__ parent,
                                const uint2* __restrict__ lo, const uint2* __restrict__ hi,
-                               const int2* __restrict__ cnt_bad, float4* __restrict__ plates, int* __restrict__ plate_id,
+                               const int2* __restrict__ cnt_bad, const unsigned* __restrict__ len,
+                               const float* __restrict__ area2, float4* __restrict__ plates, int* __restrict__ plate_id,
                                int* __restrict__ nplate) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nt) return;
     int id = -1;
-    if (parent[k] == k && cnt_bad[k].x >= kPlateMinTris && !cnt_bad[k].y) {
+    if (parent[k] == k && cnt_bad[k].x >= kPlateMinTris && !cnt_bad[k].y &&
+        area2[k] < 3.f * (unordered(hi[k].x) - unordered(lo[k].x)) * (unordered(hi[k].y) - unordered(lo[k].y))) {
         id = atomicAdd(nplate, 1);
         if (id < kMaxPlates) {
             const Flat f = flat_of(tri, k);
@@ -252,7 +270,7 @@ __global__ void k_plate_select(const float4* __restrict__ tri, int nt, const int
             a[i] = unordered(lo[k].x); a[j] = unordered(lo[k].y);
             b[i] = unordered(hi[k].x); b[j] = unordered(hi[k].y);
             plates[2 * id] = make_float4(a[0], a[1], a[2], __int_as_float(f.axis));
-            plates[2 * id + 1] = make_float4(b[0], b[1], b[2], 0.f);
+            plates[2 * id + 1] = make_float4(b[0], b[1], b[2], sqrtf(__uint_as_float(len[k])));
         } else {
             id = -1;
         }
@@ -260,17 +278,17 @@ __global__ void k_plate_select(const float4* __restrict__ tri, int nt, const int
     plate_id[k] = id;
 }
 
-// plate_of: the plate of each triangle by its input index, -1 = none.  A
-// triangle of no plate (loose) marks its leaf and every node above it.
+// place: each triangle's sorted position and plate (-1 = none) by its input
+// index.  A triangle of no plate (loose) marks its leaf and every node above it.
 __global__ void k_plate_mark(const float4* __restrict__ tri, int nt, int* __restrict__ parent,
                              const int* __restrict__ plate_id, const int* __restrict__ parent_leaf,
-                             const int* __restrict__ parent_int, int* __restrict__ plate_of,
+                             const int* __restrict__ parent_int, int2* __restrict__ place,
                              int* __restrict__ leaf_loose, int* __restrict__ node_loose, int* __restrict__ nloose) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     int plate = 0;
     if (k < nt) {
         plate = parent[k] >= 0 ? plate_id[set_root(parent, k)] : -1;
-        plate_of[__float_as_int(tri[3 * (size_t)k].w)] = plate;
+        place[__float_as_int(tri[3 * (size_t)k].w)] = make_int2(k, plate);
         leaf_loose[k] = plate < 0;
         if (plate < 0 && nt > 1)
             for (int p = parent_leaf[k]; p >= 0 && !*reinterpret_cast<volatile int*>(&node_loose[p]); p = parent_int[p])
@@ -284,7 +302,7 @@ __global__ void k_plate_mark(const float4* __restrict__ tri, int nt, int* __rest
 // not itself lie in; such a patch takes no plate for an occluder (the search
 // decides, which knows the excluded triangles).
 __global__ void k_plate_patches(const float4* __restrict__ ps, const int2* __restrict__ pe, int np, int nt,
-                                const int* __restrict__ plate_of, const float4* __restrict__ plates,
+                                const int2* __restrict__ place, const float4* __restrict__ plates,
                                 uint32_t* __restrict__ flags) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     bool flag = false;
@@ -292,7 +310,7 @@ __global__ void k_plate_patches(const float4* __restrict__ ps, const int2* __res
         const float4 s = ps[j];
         const int ex[2] = {pe[j].x, pe[j].y};
         for (int q = 0; q < 2; ++q) {
-            const int id = ex[q] >= 0 && ex[q] < nt ? plate_of[ex[q]] : -1;
+            const int id = ex[q] >= 0 && ex[q] < nt ? place[ex[q]].y : -1;
             if (id < 0) continue;
             const float4 lo = plates[2 * id];
             const int a = __float_as_int(lo.w);
@@ -317,7 +335,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Bytes of find_plates' workspace.
 size_t plates_work_bytes(int64_t nt) {
-    return align256(sizeof(int2) * (size_t)table_slots(nt)) + 4 * align256(sizeof(int) * (size_t)nt) +
+    return align256(sizeof(int2) * (size_t)table_slots(nt)) + 5 * align256(sizeof(int) * (size_t)nt) +
            3 * align256(sizeof(int2) * (size_t)nt);
 }
 
@@ -335,22 +353,23 @@ void find_plates(uvc_scene* sc, const int* parent_leaf, const int* parent_int, i
     int* parent = reinterpret_cast<int*>(take(sizeof(int) * (size_t)nt));
     unsigned* state = reinterpret_cast<unsigned*>(take(sizeof(int) * (size_t)nt));
     int* plate_id = reinterpret_cast<int*>(take(sizeof(int) * (size_t)nt));
-    int* plate_of = reinterpret_cast<int*>(take(sizeof(int) * (size_t)nt));
     uint2* lo = reinterpret_cast<uint2*>(take(sizeof(uint2) * (size_t)nt));
     uint2* hi = reinterpret_cast<uint2*>(take(sizeof(uint2) * (size_t)nt));
     int2* cnt_bad = reinterpret_cast<int2*>(take(sizeof(int2) * (size_t)nt));
+    unsigned* len = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * (size_t)nt));
+    float* area2 = reinterpret_cast<float*>(take(sizeof(float) * (size_t)nt));
     cudaMemsetAsync(table, 0xff, sizeof(int2) * (size_t)slots, stream);
     cudaMemsetAsync(lo, 0xff, sizeof(uint2) * (size_t)nt, stream);
-    cudaMemsetAsync(hi, 0, (char*)(cnt_bad + nt) - (char*)hi, stream);   // hi and cnt_bad
+    cudaMemsetAsync(hi, 0, (char*)(area2 + nt) - (char*)hi, stream);   // hi, cnt_bad, len, area2
     k_plate_init<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, state);
     k_plate_edges<<<grid(4 * (int64_t)nt), 256, 0, stream>>>(sc->tri, nt, table, slots - 1, parent, state);
-    k_plate_stats<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, state, lo, hi, cnt_bad);
+    k_plate_stats<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, state, lo, hi, cnt_bad, len, area2);
     k_plate_check<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, state, lo, hi, cnt_bad);
-    k_plate_select<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, lo, hi, cnt_bad, sc->plates, plate_id, counts);
-    k_plate_mark<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, plate_id, parent_leaf, parent_int, plate_of,
+    k_plate_select<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, lo, hi, cnt_bad, len, area2, sc->plates, plate_id, counts);
+    k_plate_mark<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, plate_id, parent_leaf, parent_int, sc->tri_place,
                                                leaf_loose, node_loose, counts + 1);
     if (np > 0)
-        k_plate_patches<<<grid(np), 256, 0, stream>>>(sc->patch_s, sc->patch_excl, np, nt, plate_of, sc->plates,
+        k_plate_patches<<<grid(np), 256, 0, stream>>>(sc->patch_s, sc->patch_excl, np, nt, sc->tri_place, sc->plates,
                                                       reinterpret_cast<uint32_t*>(sc->plates + 2 * kMaxPlates));
 }
 

@@ -18,7 +18,10 @@
 namespace uvc {
 namespace {
 
-constexpr int kAreaCandPerTask = 4;
+// Candidates per task: a patch's check points are prepared once per task, so
+// long tasks where there are enough of them (8 per resident warp keep the last
+// wave short), at least kAreaCandMin.
+constexpr int kAreaCandMin = 4, kAreaCandMax = 32;
 constexpr float kPull = 1e-3f;
 
 // v = a - o as an exact pair (hi, lo) (TwoSum).
@@ -104,6 +107,54 @@ __device__ __forceinline__ int used_triangles(const float* g, bool valid) {
     return mask;
 }
 
+// In-plane distance^2 from p to segment ab.
+__device__ __forceinline__ float seg_d2(float2 p, float2 a, float2 b) {
+    const float ux = b.x - a.x, uy = b.y - a.y, L = ux * ux + uy * uy;
+    const float t = L > 0.f ? fminf(fmaxf(((p.x - a.x) * ux + (p.y - a.y) * uy) / L, 0.f), 1.f) : 0.f;
+    const float dx = a.x + t * ux - p.x, dy = a.y + t * uy - p.y;
+    return dx * dx + dy * dy;
+}
+
+// The free distance around a check point in its own plane (PlateLane::gap):
+// from p to the border of the patch's excluded triangles, which no other
+// triangle of their plate covers.  Both triangles lie in the plane and plate of
+// the caller's choice (`in`, by triangle); 0 where p lies in neither.  Without
+// it every search to a check point ended in a walk down to the plane it lies
+// in, each neighbouring triangle tested against every source (15.2 ms per 100
+// ward candidates).
+__device__ __forceinline__ float excluded_gap(float2 p, const float2 (&T)[2][3], const bool (&in)[2]) {
+    float best = 0.f;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        if (!in[t]) continue;
+        const float2 a = T[t][0], b = T[t][1], c = T[t][2];
+        const float e0 = (b.x - a.x) * (p.y - a.y) - (b.y - a.y) * (p.x - a.x);
+        const float e1 = (c.x - b.x) * (p.y - b.y) - (c.y - b.y) * (p.x - b.x);
+        const float e2 = (a.x - c.x) * (p.y - c.y) - (a.y - c.y) * (p.x - c.x);
+        if (!((e0 > 0.f && e1 > 0.f && e2 > 0.f) || (e0 < 0.f && e1 < 0.f && e2 < 0.f))) continue;
+        // the edges of t, and of the other triangle if they share one, but that one
+        float d = 3.0e38f;
+        bool joined = false;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int k = s == 0 ? t : 1 - t, o = 1 - k;
+            if (s == 1 && !joined) break;
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                const float2 u = T[k][e], v = T[k][(e + 1) % 3];
+                int same = 0;
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    same += (T[o][q].x == u.x && T[o][q].y == u.y) || (T[o][q].x == v.x && T[o][q].y == v.y);
+                if (in[o] && same == 2) joined = true;
+                else d = fminf(d, seg_d2(p, u, v));
+            }
+        }
+        best = fmaxf(best, d);
+    }
+    return 0.95f * sqrtf(best);   // less its own rounding
+}
+
 // One packet query from o to each lane's point p (lanes in `want`); returns
 // the lanes found occluded and ORs failed lanes into `failed_all`.
 __device__ __forceinline__ uint32_t packet_to(const SceneView& S, float ox, float oy, float oz, float3 p, int2 ex,
@@ -137,14 +188,14 @@ __device__ __forceinline__ uint32_t packet_to(const SceneView& S, float ox, floa
 template <bool WEDGE>
 __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
     k_area_mean(SceneView S, const float* __restrict__ cand, int nc, LampDev L, const float* __restrict__ ptri,
-                float* __restrict__ A, int64_t lda, uint8_t* __restrict__ nclosed) {
+                float* __restrict__ A, int64_t lda, uint8_t* __restrict__ nclosed, const int2* __restrict__ tri_place, int cpt) {
     extern __shared__ __align__(16) int smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int* stack = smem + warp * S.stack_cap;
     WedgeSmem ws;
     if (WEDGE) ws = wedge_smem(reinterpret_cast<char*>(smem) + stack_smem_bytes(S.stack_cap), L.K, warp);
     const int njb = (S.np + 31) >> 5;
-    const int nchunk = (nc + kAreaCandPerTask - 1) / kAreaCandPerTask;
+    const int nchunk = (nc + cpt - 1) / cpt;
     const int64_t ntask = (int64_t)nchunk * njb;
     for (int64_t task = (int64_t)blockIdx.x * kWarpsPerBlock + warp; task < ntask;
          task += (int64_t)gridDim.x * kWarpsPerBlock) {
@@ -152,12 +203,43 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
         const int j = jb * 32 + lane;
         const PatchLane P = load_patch(S, j);
         const float* g = ptri + 18 * (size_t)(P.valid ? j : 0);
-        const bool flagged = WEDGE && S.nplate != 0 && plate_flag(S, jb, lane);
+        const PlateLane pl = WEDGE && S.nplate != 0 ? plate_lane(S, jb, lane, P) : no_plate_lane();
         const int tmask = used_triangles(g, P.valid);
         const float inv_area = P.valid && P.s.w > 0.f ? __frcp_rn(P.s.w) : 0.f;
         int cache = -1;
-        const int i1 = min(nc, (ic + 1) * kAreaCandPerTask);
-        for (int i = ic * kAreaCandPerTask; i < i1; ++i) {
+        // the check points' gaps, where plates are in use and the patch and its
+        // excluded triangles lie in one axis plane
+        float gap[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        PlateLane plc = pl;
+        plc.plate = -1;
+        if (WEDGE && S.nplate != 0 && L.plates && pl.own_axis >= 0) {
+            float2 T[2][3];
+            bool in[2] = {false, false};
+            const int ax = pl.own_axis;
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const int id = t ? P.ex.y : P.ex.x;
+                const int2 place = id >= 0 ? __ldg(&tri_place[id]) : make_int2(0, -1);
+                bool flat = place.y >= 0 && (plc.plate < 0 || plc.plate == place.y);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const float4 v = flat ? __ldg(&S.tri[3 * (size_t)place.x + q]) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    T[t][q] = ax == 0 ? make_float2(v.y, v.z) : (ax == 1 ? make_float2(v.x, v.z) : make_float2(v.x, v.y));
+                    flat = flat && pick(v.x, v.y, v.z, ax) == pl.own;
+                }
+                in[t] = flat;
+                if (flat) plc.plate = place.y;
+            }
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                if (!((tmask >> (q / 3)) & 1)) continue;
+                const float3 v = pulled(vertex(g, q), P.s);
+                if (pick(v.x, v.y, v.z, ax) == pl.own)
+                    gap[q] = excluded_gap(ax == 0 ? make_float2(v.y, v.z) : (ax == 1 ? make_float2(v.x, v.z) : make_float2(v.x, v.y)), T, in);
+            }
+        }
+        const int i1 = min(nc, (ic + 1) * cpt);
+        for (int i = ic * cpt; i < i1; ++i) {
             const float cx = __ldg(&cand[3 * (size_t)i]), cy = __ldg(&cand[3 * (size_t)i + 1]),
                         cz = __ldg(&cand[3 * (size_t)i + 2]);
             float E = 0.f;
@@ -171,6 +253,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
                 // q = -1: the centroid; q = 0..5: the check points.  One call site of
                 // the (large, inlined) wedge search keeps the kernel's code small.
                 for (int q = -1; q < 6; ++q) {
+                    PlateLane plq = q < 0 ? pl : plc;
                     uint32_t want_q = want;
                     float szq = P.s.z, gxq = gx, gyq = gy, lq = lend, dq = dmax;
                     if (q >= 0) {
@@ -183,10 +266,13 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
                         if (want_q) wedge_setup_point(L, cx, cy, cz, pq, want_q, dq, gxq, gyq);
                         szq = pq.z;
                         lq = 1.f;
+                        plq.gap = 0.f;
+#pragma unroll
+                        for (int k = 0; k < 6; ++k) plq.gap = q == k ? gap[k] : plq.gap;   // no indexed registers
+                        if (!(plq.gap > 0.f)) plq.own_axis = -1;
                     }
                     uint32_t fq;
-                    const uint32_t oc = wedge_search<false>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex,
-                                                            flagged, lane, stack, ws, cache, fq, nullptr);
+                    const uint32_t oc = wedge_search<false>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex, plq, lane, stack, ws, cache, fq, nullptr);
                     failed_all |= fq;
                     if (q < 0) {
                         vis_c = ((fq >> lane) & 1u) ? 0u : (facing & ~oc);
@@ -290,16 +376,18 @@ int irradiance_area_mean(const uvc_scene* sc, const float* cand, int64_t nc, con
         if (e != cudaSuccess) return status_from_cuda(e);
     }
     const int njb = (S.np + 31) / 32;
-    const int64_t ntask = ((nc + kAreaCandPerTask - 1) / kAreaCandPerTask) * njb;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     int grid = per_sm * sm_count();
+    const int64_t per_warp = nc * njb / ((int64_t)grid * kWarpsPerBlock);   // candidates x patch blocks
+    const int cpt = (int)std::max<int64_t>(kAreaCandMin, std::min<int64_t>(kAreaCandMax, per_warp / 8));
+    const int64_t ntask = ((nc + cpt - 1) / cpt) * njb;
     if ((int64_t)grid * kWarpsPerBlock > ntask) grid = (int)((ntask + kWarpsPerBlock - 1) / kWarpsPerBlock);
     if (wedge)
-        k_area_mean<true><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, ptri, A, lda, nclosed);
+        k_area_mean<true><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, ptri, A, lda, nclosed, sc->tri_place, cpt);
     else
-        k_area_mean<false><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, ptri, A, lda, nclosed);
+        k_area_mean<false><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, ptri, A, lda, nclosed, sc->tri_place, cpt);
     return status_from_cuda(cudaGetLastError());
 }
 

@@ -418,15 +418,18 @@ __device__ __forceinline__ PatchLane load_patch(const SceneView& S, int j) {
 //             of the plane, or crosses it well outside: none of them hits
 //   open      anything nearer to a border or an end; only these segments go
 //             on to the search
-// so every visibility bit is the search's own.  "Well": the test's rounding
-// moves a triangle, seen along the segment, by about 2^-22 of the distances
-// involved (subtractions 2^-24, shear 2^-23); the margin is 8 times that, and
-// divided by the segment's cosine with the plane's normal within the plane.
-// Off the plane 2^-14 of the distances is asked for: the rounding of a
-// triangle's barycentric coordinates (2^-22 times its 1 : 32 at most, over the
-// cosine) moves a hit by that part of its length along the segment, 2^-17 of
-// it along the normal.  Both are taken of the scene's diagonal plus the
-// longest segment.  NaN and infinities fail the comparisons and stay open.
+// so every visibility bit is the search's own.  "Well": with u = 2^-24 and R the
+// distance of a triangle's vertices from the source, the test's roundings move
+// the triangle, seen along the segment, by at most 6 u R per coordinate
+// (differences u, shear 4 u, product u), 2^-20.9 R in all.  R is at most the
+// longest segment plus the plate's longest triangle edge for the triangles
+// near a crossing; the margin is 2^-19 of that sum, divided by the segment's
+// cosine with the plane's normal within the plane.  Off the plane the ends must
+// be by 2^-19 of that sum plus 2^-16 of the edge: the rounding of a triangle's
+// barycentric coordinates (2 u edge^2 each over its projected area, at least
+// edge^2 / 32 times the cosine: 192 u / cosine in all) moves a hit by that part
+// of its edge along the segment, 192 u of it along the normal.  NaN and
+// infinities fail the comparisons and stay open.
 //
 // Which plates the packet's wedges can reach is found 32 at a time, a plate
 // per lane, against the packet's shaft: the hull's box, the two vertical
@@ -471,6 +474,26 @@ __device__ __forceinline__ Slabs slabs_of(float cx, float cy, float gx, float gy
     return b;
 }
 
+// What the plates need to know of the lane's point.  A point exactly in a
+// plate's plane, with no other triangle of that plane (excluded ones aside)
+// nearer than `gap`: a segment from the free side meets the plane in the point
+// only.  The test's roundings along the normal scale with the source's height
+// over the plane here, as the point and the vertices share that coordinate:
+// seen in the plane they move a triangle by at most 6 u (dmax + edge) whatever
+// the angle.  A point outside a triangle by more lies outside the moved one, and
+// past one of its edges by 1/64 of that or more (angles of 1/32 at least), which
+// the products' rounding (2 u edge) cannot hide: clear from 2^-20 dmax + 2^-16
+// edge on.
+struct PlateLane {
+    bool flagged;    // takes no plate for an occluder (plates.cu: k_plate_patches)
+    int own_axis;    // axis of the point's own plane, -1 = none
+    float own;       // its coordinate
+    float gap;       // metres
+    int plate;       // the only plate that the gap holds for, -1 = all of the plane
+};
+
+__device__ __forceinline__ PlateLane no_plate_lane() { return PlateLane{false, -1, 0.f, 0.f, -1}; }
+
 // The sources q < K of a column stand at (cx, cy, zsrc(q)); `want` holds the
 // lane's sources that need a search, zlo and zhi their extreme heights, g and
 // sz the lane's point (from c, horizontally; height), lend the largest
@@ -480,14 +503,12 @@ __device__ __forceinline__ Slabs slabs_of(float cx, float cy, float gx, float gy
 template <class Z>
 __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, int K, float cx, float cy, float sz,
                                                   float gx, float gy, float zlo, float zhi, float lend, float dmax,
-                                                  const Slabs& sl, bool flagged, int lane, uint32_t& want) {
+                                                  const Slabs& sl, const PlateLane& pl, int lane, uint32_t& want) {
     const float kBig = 3.0e38f;
     const bool a0 = want != 0u;
     const float delta = S.cut_eps, diag = S.cut_eps * 1e5f;
     // far outside the scene (or infinite, or NaN) the widening no longer covers the rounding of the shaft
     if (__any_sync(kFull, a0 && !(dmax < 32.f * diag))) return want;
-    const float far_off = (diag + dmax) * 6.103515625e-05f;       // 2^-14
-    const float near_in = (diag + dmax) * 1.9073486328125e-06f;   // 2^-19
     // the packet's shaft, relative to the column's foot in x and y
     const float tx = lend * gx, ty = lend * gy;
     const float tl = fmaf(lend, sz - zlo, zlo), th = fmaf(lend, sz - zhi, zhi);
@@ -527,6 +548,9 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
             const int p = base + __ffs(hits) - 1;
             const float4 lo = __ldg(&S.plates[2 * p]), hi = __ldg(&S.plates[2 * p + 1]);
             const int axis = __float_as_int(lo.w);
+            const float reach = dmax + hi.w;
+            const float far_off = reach * 1.9073486328125e-06f + hi.w * 1.52587890625e-05f;   // 2^-19, 2^-16
+            const float near_in = reach * 1.9073486328125e-06f;   // 2^-19
             if (want) {
                 // the wedge box test (wedge_pair_hits) on the rectangle's box
                 const bool nx = __float_as_uint(gx) >> 31, ny = __float_as_uint(gy) >> 31;
@@ -536,7 +560,12 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
                 const float wh = fmaxf(fmaf(a, sz - zhi, zhi), fmaf(b, sz - zhi, zhi)) + delta;
                 if (a <= b && hi.z >= wl && lo.z <= wh) {
                     uint32_t blocked = 0u, clear = 0u;
-                    if (axis != 2) {
+                    if (axis == pl.own_axis && pl.own == (axis == 0 ? lo.x : (axis == 1 ? lo.y : lo.z)) &&
+                        (pl.plate < 0 || pl.plate == p)) {
+                        const float h = axis == 0 ? fabsf(cx - lo.x) : (axis == 1 ? fabsf(cy - lo.y) : fmaxf(zlo - lo.z, lo.z - zhi));
+                        if (pl.gap > 9.5367431640625e-07f * dmax + 1.52587890625e-05f * hi.w && h > 1e-6f * reach)
+                            clear = want;   // 2^-20, 2^-16
+                    } else if (axis != 2) {
                         const bool isx = axis == 0;
                         const float ho = isx ? cx - lo.x : cy - lo.y, ga = isx ? gx : gy, ig = isx ? sl.igx : sl.igy;
                         const float gb = isx ? gy : gx, hs = ho + ga;
@@ -571,7 +600,7 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
                                 }
                             }
                     }
-                    if (flagged) blocked = 0u;
+                    if (pl.flagged) blocked = 0u;
                     open |= want & ~(blocked | clear);
                     want &= ~blocked;
                 }
@@ -582,9 +611,20 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
     return open & want;
 }
 
-// Flag word bit of the lane's patch (plates.cu: k_plate_patches).
-__device__ __forceinline__ bool plate_flag(const SceneView& S, int jb, int lane) {
-    return (__ldg(reinterpret_cast<const uint32_t*>(S.plates + 2 * kMaxPlates) + jb) >> lane) & 1u;
+// The lane's patch (its flag bit: plates.cu, k_plate_patches).  A patch on an
+// axis plane that has a clearance has no triangle of that plane but its own
+// within 2^-14 of the scene's diagonal (build_bvh.cu: k_clearance).
+__device__ __forceinline__ PlateLane plate_lane(const SceneView& S, int jb, int lane, const PatchLane& P) {
+    PlateLane pl;
+    pl.flagged = (__ldg(reinterpret_cast<const uint32_t*>(S.plates + 2 * kMaxPlates) + jb) >> lane) & 1u;
+    const bool x = fabsf(P.n.x) == 1.f, y = fabsf(P.n.y) == 1.f, z = fabsf(P.n.z) == 1.f;
+    const bool unit = (x && P.n.y == 0.f && P.n.z == 0.f) || (y && P.n.x == 0.f && P.n.z == 0.f) ||
+                      (z && P.n.x == 0.f && P.n.y == 0.f);
+    pl.own_axis = unit && P.n.w > 0.f ? (x ? 0 : (y ? 1 : 2)) : -1;
+    pl.own = x ? P.s.x : (y ? P.s.y : P.s.z);
+    pl.gap = S.cut_eps * 6.f;   // 1e5 2^-14 = 6.1
+    pl.plate = -1;
+    return pl;
 }
 
 // Irradiance of candidate i at this lane's patch (lanes beyond np give 0).
@@ -605,7 +645,7 @@ __device__ __forceinline__ float irradiance_entry(const SceneView& S, const floa
     const float cx = __ldg(&cand[3 * (size_t)i]), cy = __ldg(&cand[3 * (size_t)i + 1]),
                 cz = __ldg(&cand[3 * (size_t)i + 2]);
     const bool plates = !COUNT && S.nplate != 0 && L.plates;
-    const bool flagged = plates && plate_flag(S, jb, lane);
+    const PlateLane pl = plates ? plate_lane(S, jb, lane, P) : no_plate_lane();
     float E = 0.f;
     bool bad = false;
     for (int m = 0; m < L.K; ++m) {
@@ -623,7 +663,7 @@ __device__ __forceinline__ float irradiance_entry(const SceneView& S, const floa
         const uint32_t before = want;
         if (plates && __any_sync(kFull, want))
             open = plates_decide(S, [&](int) { return oz; }, 1, ox, oy, s4.z, -hx, -hy, oz, oz,
-                                 tend, d, slabs_of(ox, oy, -hx, -hy, S.cut_eps), flagged, lane, want);
+                                 tend, d, slabs_of(ox, oy, -hx, -hy, S.cut_eps), pl, lane, want);
         for (int whole = plates && (S.nplate & kLooseBit) ? 0 : 1; whole < 2; ++whole) {
             const uint32_t search = __ballot_sync(kFull, want && (whole ? open : !open));
             if (!search) continue;
@@ -1161,7 +1201,7 @@ __device__ __forceinline__ void wedge_shear(const LampDev& L, float cz, float sz
 template <bool COUNT>
 __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampDev& L, float cx, float cy, float cz,
                                                  float sz, float gx, float gy, uint32_t want, float lend, float dmax,
-                                                 int2 ex, bool flagged, int lane, int* stack, const WedgeSmem& ws,
+                                                 int2 ex, const PlateLane& pl, int lane, int* stack, const WedgeSmem& ws,
                                                  int& cache, uint32_t& failed, unsigned long long* ctr) {
     failed = 0;
     if (S.nt == 0 || !__any_sync(kFull, want != 0u)) return 0u;
@@ -1182,7 +1222,7 @@ __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampD
             }
         }
         open = plates_decide(S, [&](int q) { return __fadd_rn(cz, L.oz[q]); }, L.K, cx, cy, sz, gx, gy, zlo, zhi, lend,
-                             dmax, sl, flagged, lane, want);
+                             dmax, sl, pl, lane, want);
     }
     for (int whole = plates && (S.nplate & kLooseBit) ? 0 : 1; whole < 2; ++whole) {
         uint32_t set = want & (whole ? open : ~open);
@@ -1274,8 +1314,8 @@ __device__ __forceinline__ float irradiance_wedge(const SceneView& S, const floa
     float E;
     const uint32_t facing = wedge_setup_patch(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, E);
     uint32_t failed;
-    const bool flagged = !COUNT && S.nplate != 0 && plate_flag(S, jb, lane);
-    const uint32_t occl = wedge_search<COUNT>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, flagged, lane,
+    const PlateLane pl = !COUNT && S.nplate != 0 ? plate_lane(S, jb, lane, P) : no_plate_lane();
+    const uint32_t occl = wedge_search<COUNT>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, pl, lane,
                                               stack, ws, cache, failed, ctr);
     const bool bad = (failed >> lane) & 1u;
     const uint32_t visible = bad ? 0u : (facing & ~occl);

@@ -96,7 +96,8 @@ struct uvc_scene {
     float4* patch_n = nullptr;    // [np] (normal, clearance): see k_clearance
     int2* patch_excl = nullptr;   // [np]
     float* area_total = nullptr;  // [1]
-    float4* plates = nullptr;     // [kMaxPlates][2]: (lo, axis bits), (hi, 0); then one flag bit per patch
+    float4* plates = nullptr;     // [kMaxPlates][2]: (lo, axis bits), (hi, longest triangle edge); then one flag bit per patch
+    int2* tri_place = nullptr;    // [nt] by input index: (sorted position, plate or -1)
     int32_t nplate = 0;
     int32_t nloose = 0;           // triangles of no plate
     int* status = nullptr;        // [1] device status word (0 = ok)

@@ -11,10 +11,11 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2103_14137_gb300 as uvc
 from synth.scenes import Lamp, line_lamp, point_lamp
-from tests.gpu_util import build_arrays
-from tests.test_gpu_wedge import _same_as_per_source
+from tests.gpu_util import build_arrays, lamp_of
+from tests.test_gpu_wedge import _area, _same_as_per_source
 
 pytestmark = pytest.mark.gpu
 
@@ -79,9 +80,9 @@ def _lamps():
     return {"line2": line_lamp(0.5, 2, 60.0), "line16": line_lamp(1.2, 16, 120.0), "point": point_lamp(80.0), "tube": tube}
 
 
-@pytest.mark.parametrize("name", list(_scenes()))
-def test_plates_give_the_search_results(name):
-    T, loose = _scenes()[name]
+def _patches(T, name):
+    """The scene's arrays and 300 patches on its triangles: (verts, tris, points, normals, excl), and the
+    patches' own triangles."""
     verts, inv = np.unique(T.reshape(-1, 3).astype(np.float32), axis=0, return_inverse=True)
     tris = inv.reshape(-1, 3).astype(np.int32)
     rng = np.random.default_rng(len(name))
@@ -102,9 +103,45 @@ def test_plates_give_the_search_results(name):
     cand[:8, 0] = [1.0, 2.0, 2.5, 3.0, 0.5, 1.5, 2.25, 1.0]            # in the planes of faces, above their edges
     cand[:8, 1] = [0.5, 1.0, 1.25, 2.0, 2.0, 0.75, 0.5, 2.0]
     cand[8:12, 2] = [0.25, 0.5, 0.75, 1.0]
-    sc = build_arrays(verts, tris, cen, nrm, np.ones(own.size, np.float32), excl)
+    return (verts, tris, cen, nrm, excl), V[own].astype(np.float32), cand
+
+
+@pytest.mark.parametrize("name", list(_scenes()))
+def test_plates_give_the_search_results(name):
+    T, loose = _scenes()[name]
+    arrays, _, cand = _patches(T, name)
+    sc = build_arrays(*arrays[:4], np.ones(300, np.float32), arrays[4])
     assert (uvc.scene_export_traversal(sc)["nodes4"][0, 30] != 0) == loose
-    for lname, L in _lamps().items():
-        _same_as_per_source((verts, tris, cen, nrm, excl), sc, cand, L)
+    for L in _lamps().values():
+        _same_as_per_source(arrays, sc, cand, L)
     torch.cuda.synchronize()
+    sc.free()
+
+
+@pytest.mark.parametrize("name", ["plates_only", "window_in_a_wall", "doubled_triangle", "over_32_plates"])
+@pytest.mark.parametrize("lamp", ["line2", "line16"])
+def test_area_mean_at_plates_gives_the_search_results(name, lamp):
+    """Check points, too, are decided at plates: patches that are their excluded triangle, the half of it, a
+    part reaching outside of it, and patches that exclude nothing."""
+    T, _ = _scenes()[name]
+    arrays, own, cand = _patches(T, name)
+    verts, tris, cen, nrm, excl = arrays
+    s = cen[:, None, :]
+    ptri = np.zeros((300, 2, 3, 3), np.float32)
+    ptri[:, 0] = own
+    ptri[1::4, 0, 2] = 0.5 * (own[1::4, 1] + own[1::4, 2])
+    ptri[2::4, 0] = s[2::4] + 1.5 * (own[2::4] - s[2::4])
+    excl[3::4, 0] = -1
+    area = np.full(300, 0.1, np.float32)
+    sc = build_arrays(verts, tris, cen, nrm, area, excl)
+    L = _lamps()[lamp]
+    Aw, cw = _area(sc, cand, lamp_of(L), ptri, True)
+    Ap, cp = _area(sc, cand, lamp_of(L), ptri, False)
+    differ = ((Aw != Ap) | (cw != cp)).cpu().numpy()
+    if differ.any():
+        pairs = np.argwhere(differ)
+        _, _, flag = oracle.area_mean(verts, tris, cen, nrm, area, excl, ptri, cand, L.offsets, L.weights, L.power,
+                                      pairs=pairs)
+        assert np.all(flag != 0), f"{int((flag == 0).sum())} of {pairs.shape[0]} differing pairs are not grazing"
+    assert (cw > 0).any()
     sc.free()
