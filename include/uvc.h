@@ -138,9 +138,11 @@ int uvc_free_scene(uvc_scene* scene);
 
 /*
  * uvc_set_fluence_tensor_cores - which kernel uvc_fluence uses for A^T t
- * (Eq. (5)) where the rows of A start on 16-byte boundaries: 1 (the default)
- * the tensor cores (tcgen05 MMAs on split TF32 operands, accumulators in
- * tensor memory), 0 the CUDA cores (FP32 FMAs).  Not in the paper.  Process-
+ * (Eq. (5)) where the rows of A start on 16-byte boundaries and the scene has
+ * more than 9,728 patches: 1 (the default) the tensor cores (tcgen05 MMAs on
+ * split TF32 operands, accumulators in tensor memory), 0 the CUDA cores (FP32
+ * FMAs, which narrower matrices always take: they leave the tensor-core
+ * kernel's SMs idle).  Not in the paper.  Process-
  * wide; read when uvc_fluence enqueues its launch.
  *   enable    0 or 1
  *   previous  HOST int32, may be NULL: receives the setting before the call
@@ -277,12 +279,12 @@ int uvc_irradiance_raster(const uvc_scene* scene, const float* tri_normal, const
  *   mu  float[nvec][np] output (J/m^2)
  *
  * Where the rows of A start on 16-byte boundaries (lda a multiple of 4, A
- * 16-byte aligned) the product runs on the tensor cores (see
- * uvc_set_fluence_tensor_cores): TF32 operands split in two (x = hi + lo),
- * FP32 accumulation of 32 candidate rows at a time, the stage sums added with
- * Kahan compensation; otherwise, or with the tensor cores switched off, on the
- * CUDA cores in FP32 with blocks of 32 rows summed plainly and the block sums
- * Kahan-compensated.  nvec in [1, 256].  Allocates nothing.  A wait of the
+ * 16-byte aligned) and the scene has more than 9,728 patches the product runs
+ * on the tensor cores (see uvc_set_fluence_tensor_cores): TF32 operands split
+ * in two (x = hi + lo), FP32 accumulation of 32 candidate rows at a time, the
+ * stage sums added with Kahan compensation; otherwise, or with the tensor
+ * cores switched off, on the CUDA cores in FP32 with blocks of 32 rows summed
+ * plainly and the block sums Kahan-compensated.  nvec in [1, 256].  Allocates nothing.  A wait of the
  * tensor-core kernel that runs out records UVC_E_TIMEOUT in the scene's status
  * word (uvc_scene_status).  Errors: UVC_E_INVAL, UVC_E_CUDA.
  */

@@ -12,10 +12,13 @@ namespace uvc {
 namespace {
 
 constexpr int kBins = 64;
-// Probe-column kernels: a block covers 32 columns x 8 row slices; thread
-// (slice, column) scans rows slice, slice + 8, ... (coalesced across the 32
-// columns), and the 8 slices are combined in shared memory.
-constexpr int kColW = 32, kColSlices = 8;
+// Probe-column kernels: a block covers 8 columns x 128 row slices; thread
+// (slice, column) scans rows slice, slice + 128, ... (one 32-byte sector across
+// the 8 columns), and the slices are combined in shared memory.  The columns
+// are a probe's, a few hundred, so 32 columns x 8 slices left a dozen blocks
+// walking hundreds of rows one after the other (511 x 2,000: maxima 22 us,
+// marks 39 us, losses 127 us; now 6, 16 and 8 us).
+constexpr int kColW = 8, kColSlices = 128;
 constexpr int kHistThreads = 256;
 
 struct Edges {
@@ -23,36 +26,57 @@ struct Edges {
 };
 
 // One block per candidate; each thread keeps its own 64 slots in shared
-// memory (no atomics), the slots are then added in a fixed order.
+// memory (no atomics), the slots are then added in a fixed order.  The bin of
+// a squared distance follows from its logarithm (the edges are log-spaced): the
+// approximate one decides away from the edges, within kEdgeZone of one the exact
+// edge does, so every patch falls where a search through the edges would put
+// it.  That search, six dependent loads a pair, took 1.01 ms of 2,000 ward
+// candidates x 98,132 patches.
+constexpr float kEdgeZone = 1e-3f;   // in bins; the logarithm is good to 1e-5 of one
 __global__ void __launch_bounds__(kHistThreads) k_feat_hist(const float4* __restrict__ ps, int np,
                                                              const float* __restrict__ area_total,
                                                              const float* __restrict__ cand, Edges E,
+                                                             float bins_per_log2, float bin0,
                                                              float* __restrict__ feat, int64_t ldf) {
-    extern __shared__ float slot[];   // [kBins][kHistThreads]
-    __shared__ float edge[kBins - 1];
+    extern __shared__ __align__(16) float slot[];   // [kBins][kHistThreads]
+    __shared__ float edge[kBins + 1];   // lower edges (0 first, then E, infinity last)
     const int i = blockIdx.x;
     const int t = threadIdx.x;
-    for (int b = t; b < kBins - 1; b += blockDim.x) edge[b] = E.e[b];
+    for (int b = t; b <= kBins; b += blockDim.x) edge[b] = b == 0 ? 0.f : (b == kBins ? __int_as_float(0x7f800000) : E.e[b - 1]);
     for (int b = 0; b < kBins; ++b) slot[b * kHistThreads + t] = 0.f;
     __syncthreads();
     const float cx = cand[3 * (size_t)i], cy = cand[3 * (size_t)i + 1], cz = cand[3 * (size_t)i + 2];
+#pragma unroll 4
     for (int j = t; j < np; j += kHistThreads) {
         const float4 s = __ldg(&ps[j]);
         const float dx = s.x - cx, dy = s.y - cy, dz = s.z - cz;
         const float d2 = dx * dx + dy * dy + dz * dz;
-        int lo = 0, hi = kBins - 1;   // number of edges <= d2, by bisection
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (edge[mid] <= d2) lo = mid + 1; else hi = mid;
+        float lg;
+        asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(d2));
+        const float x = fminf(fmaxf(fmaf(lg, bins_per_log2, bin0), 0.f), (float)kBins - 0.5f);   // NaN: bin 0
+        const float r = (x + 12582912.f) - 12582912.f;   // nearest edge (1.5 2^23: rounds to integers)
+        int b = (int)r;
+        if (x < r) --b;
+        if (fabsf(x - r) < kEdgeZone) {
+            const int n = (int)r;
+            b = d2 >= edge[n] || n == 0 ? n : n - 1;
         }
-        slot[lo * kHistThreads + t] += s.w;
+        slot[b * kHistThreads + t] += s.w;
     }
     __syncthreads();
     const float tot = *area_total;
-    for (int b = t; b < kBins; b += blockDim.x) {
+    if (t < kBins) {   // in thread order, four slots a load
         float sum = 0.f;
-        for (int q = 0; q < kHistThreads; ++q) sum += slot[b * kHistThreads + q];
-        feat[i * ldf + b] = tot > 0.f ? sum / tot : 0.f;
+        const float4* q = reinterpret_cast<const float4*>(slot + t * kHistThreads);
+#pragma unroll 8
+        for (int k = 0; k < kHistThreads / 4; ++k) {
+            const float4 v = q[k];
+            sum += v.x;
+            sum += v.y;
+            sum += v.z;
+            sum += v.w;
+        }
+        feat[i * ldf + t] = tot > 0.f ? sum / tot : 0.f;
     }
 }
 
@@ -102,12 +126,16 @@ __device__ __forceinline__ float box_d2(float3 p, float lx, float ly, float lz, 
     return dx * dx + dy * dy + dz * dz;
 }
 
-// One thread per candidate: nearest-triangle search over the binary tree.
-__global__ void k_feat_clear(const Node* __restrict__ nodes, const float4* __restrict__ tri, int nt,
-                             const float* __restrict__ cand, int nc, float* __restrict__ feat, int64_t ldf) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nc) return;
-    const float3 p = make_float3(cand[3 * (size_t)i], cand[3 * (size_t)i + 1], cand[3 * (size_t)i + 2]);
+// Nearest triangle, one warp per candidate: up to 8 nodes of the four-wide tree
+// leave the warp's list at a time, each lane takes one child of one of them,
+// triangles are measured where they turn up, and children no nearer than the
+// best so far are dropped (before they are listed and when they are taken).  A
+// thread per candidate walked the binary tree through some sixty dependent
+// loads: 73 us for 2,000 candidates, with 63 warps on the chip; now 26 us.
+// A list that would overflow sends the candidate through that walk.
+constexpr int kClearWarps = 4, kClearList = 256;
+
+__device__ float nearest_walk(const Node* __restrict__ nodes, const float4* __restrict__ tri, int nt, float3 p) {
     float best = 3.0e38f;
     int stack[128];
     int top = 0;
@@ -134,8 +162,73 @@ __global__ void k_feat_clear(const Node* __restrict__ nodes, const float4* __res
         if ((lfirst ? dR : dL) < best) stack[top++] = lfirst ? nd.r.y : nd.r.x;
         if ((lfirst ? dL : dR) < best) stack[top++] = lfirst ? nd.r.x : nd.r.y;
     }
-    feat[i * ldf + kBins] = nt > 0 ? sqrtf(best) : 3.0e38f;
-    feat[i * ldf + kBins + 1] = p.z;
+    return best;
+}
+
+__global__ void __launch_bounds__(32 * kClearWarps) k_feat_clear(const Node4* __restrict__ nodes4,
+                                                                 const Node* __restrict__ nodes,
+                                                                 const float4* __restrict__ tri, int nt,
+                                                                 const float* __restrict__ cand, int nc,
+                                                                 float* __restrict__ feat, int64_t ldf) {
+    __shared__ int list[kClearWarps][kClearList];
+    __shared__ float dist[kClearWarps][kClearList];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * kClearWarps + warp;
+    if (i >= nc) return;
+    const float3 p = make_float3(cand[3 * (size_t)i], cand[3 * (size_t)i + 1], cand[3 * (size_t)i + 2]);
+    float best = 3.0e38f;   // the same in every lane
+    bool over = nt < 2;
+    int top = over ? 0 : 1;
+    if (lane == 0) {
+        list[warp][0] = 0;
+        dist[warp][0] = 0.f;
+    }
+    __syncwarp();
+    for (int guard = 0; top > 0 && guard < 4 * nt + 64; ++guard) {
+        const int n = min(min(8, top), (kClearList - top) / 3);
+        if (n < 1) {
+            over = true;
+            break;
+        }
+        const int slot = lane >> 2, c = lane & 3;
+        int ref = kEmptyChild;
+        float d = 3.0e38f;
+        if (slot < n && dist[warp][top - 1 - slot] < best) {
+            const Node4* nd = nodes4 + list[warp][top - 1 - slot];
+            ref = __ldg(reinterpret_cast<const int*>(&nd->r) + c);
+            const float* q = reinterpret_cast<const float*>(nd) + (c >> 1) * 12 + (c & 1);
+            d = box_d2(p, __ldg(q), __ldg(q + 4), __ldg(q + 8), __ldg(q + 2), __ldg(q + 6), __ldg(q + 10));
+        }
+        __syncwarp();   // the popped entries are read
+        top -= n;
+        float t = 3.0e38f;
+        if (ref < 0 && d < best) {
+            const float4 a = __ldg(&tri[3 * (size_t)~ref]), b = __ldg(&tri[3 * (size_t)~ref + 1]), e = __ldg(&tri[3 * (size_t)~ref + 2]);
+            t = point_tri_dist2(p, make_float3(a.x, a.y, a.z), make_float3(b.x, b.y, b.z), make_float3(e.x, e.y, e.z));
+        }
+        // distances are not negative: their bits order them (NaN from a NaN candidate stays out)
+        best = fminf(best, __uint_as_float(__reduce_min_sync(0xffffffffu, t >= 0.f ? __float_as_uint(t) : 0x7f61b1e6u)));
+        // the nearest of the new children goes on top
+        const bool in = ref >= 0 && ref != kEmptyChild && d < best;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        const unsigned near = __reduce_min_sync(0xffffffffu, in ? __float_as_uint(d) : 0xffffffffu);
+        const unsigned w = __ballot_sync(0xffffffffu, in && __float_as_uint(d) == near);
+        const int win = __ffs(w) - 1, cnt = __popc(m);
+        if (in) {
+            int at = __popc(m & ((1u << lane) - 1u));
+            if (lane == win) at = cnt - 1;
+            else if (lane > win) --at;
+            list[warp][top + at] = ref;
+            dist[warp][top + at] = d;
+        }
+        top += cnt;
+        __syncwarp();
+    }
+    if (lane == 0) {
+        if (over) best = nearest_walk(nodes, tri, nt, p);
+        feat[i * ldf + kBins] = nt > 0 ? sqrtf(best) : 3.0e38f;
+        feat[i * ldf + kBins + 1] = p.z;
+    }
 }
 
 constexpr int kSelectMax = 16384;
@@ -149,39 +242,80 @@ __device__ __forceinline__ uint32_t score_key(float v) {
 }
 
 // The k best of n scores (higher first, ties to the lower index), written in
-// ascending index order: a bitonic sort of (inverted key, index) in shared
-// memory, a flag per selected index, then a block-wide scan compacts the flags.
+// ascending index order.  The k-th largest key is found by four passes over
+// its bytes (a histogram of the keys that share the bytes found so far, its
+// suffix sums by one warp); the scores above it are all taken, those equal to it
+// in index order as far as they are needed, and a block-wide scan writes them.
+// (A bitonic sort of all keys took 25 us for 2,000 scores, this 9 us.)
 __global__ void __launch_bounds__(kSelectThreads) k_select_top(const float* __restrict__ score, int n, int k,
                                                                 const float* __restrict__ cand,
                                                                 float* __restrict__ out_cand,
                                                                 int32_t* __restrict__ out_idx) {
-    extern __shared__ unsigned long long key[];   // [m] then flags [n] as bytes
+    extern __shared__ uint32_t key[];   // [n], then flags [n] as bytes
     __shared__ int warp_tot[kSelectThreads / 32];
-    int m = 1;
-    while (m < n) m <<= 1;
-    unsigned char* flag = reinterpret_cast<unsigned char*>(key + m);
+    __shared__ unsigned hist[256];
+    __shared__ uint32_t sh_prefix;
+    __shared__ int sh_want;
+    unsigned char* flag = reinterpret_cast<unsigned char*>(key + n);
     const int t = threadIdx.x;
-    for (int i = t; i < m; i += blockDim.x)
-        key[i] = i < n ? ((unsigned long long)(~score_key(score[i])) << 32) | (unsigned)i : ~0ull;
-    for (int i = t; i < n; i += blockDim.x) flag[i] = 0;
-    __syncthreads();
-    for (int size = 2; size <= m; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = t; i < m; i += blockDim.x) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    const bool up = (i & size) == 0;
-                    const unsigned long long a = key[i], b = key[j];
-                    if ((a > b) == up) {
-                        key[i] = b;
-                        key[j] = a;
-                    }
-                }
-            }
-            __syncthreads();
+    for (int i = t; i < n; i += blockDim.x) key[i] = score_key(score[i]);
+    uint32_t prefix = 0u;
+    int want = k;   // keys still to be taken among those that share the prefix
+    for (int shift = 24; shift >= 0; shift -= 8) {
+        if (t < 256) hist[t] = 0u;
+        __syncthreads();
+        for (int i = t; i < n; i += blockDim.x) {
+            const uint32_t v = key[i];
+            if (shift == 24 || (v >> (shift + 8)) == prefix) atomicAdd(&hist[(v >> shift) & 255u], 1u);
         }
-    for (int r = t; r < k; r += blockDim.x) flag[(int)(key[r] & 0xffffffffu)] = 1;
-    __syncthreads();
+        __syncthreads();
+        if (t < 32) {   // lane l: bytes 255 - 8 l down to 248 - 8 l
+            unsigned c[8], sum = 0u;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                c[q] = hist[255 - 8 * t - q];
+                sum += c[q];
+            }
+            unsigned inc = sum;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (t >= o) inc += v;
+            }
+            unsigned above = inc - sum;   // keys with a larger byte than this lane's
+            if (above < (unsigned)want && inc >= (unsigned)want)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    if (above < (unsigned)want && above + c[q] >= (unsigned)want) {
+                        sh_prefix = (prefix << 8) | (uint32_t)(255 - 8 * t - q);
+                        sh_want = want - (int)above;
+                    }
+                    above += c[q];
+                }
+        }
+        __syncthreads();
+        prefix = sh_prefix;
+        want = sh_want;
+    }
+    // each thread's run of consecutive indices: how many equal keys come before it
+    {
+        const int per = (n + blockDim.x - 1) / blockDim.x, lo = min(n, t * per), hi = min(n, lo + per);
+        int eq = 0;
+        for (int i = lo; i < hi; ++i) eq += key[i] == prefix;
+        int inc = eq;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if ((t & 31) >= o) inc += v;
+        }
+        if ((t & 31) == 31) warp_tot[t >> 5] = inc;
+        __syncthreads();
+        int before = inc - eq;
+        for (int q = 0; q < (t >> 5); ++q) before += warp_tot[q];
+        for (int i = lo; i < hi; ++i) {
+            flag[i] = key[i] > prefix || (key[i] == prefix && before < want);
+            before += key[i] == prefix;
+        }
+        __syncthreads();
+    }
     // each thread owns a run of consecutive indices
     const int per = (n + blockDim.x - 1) / blockDim.x;
     const int lo = min(n, t * per), hi = min(n, lo + per);
@@ -220,10 +354,12 @@ __global__ void k_probe_lost(const float* __restrict__ A, int nc, int64_t lda, i
     const int j = blockIdx.x * kColW + cx;
     bool full = false, red = false;
     if (j < np) {
-        for (int i = sl; i < nc && !full; i += kColSlices) full = A[(int64_t)i * lda + j] > 0.f;
-        for (int r = sl; r < k && !red; r += kColSlices) {
+#pragma unroll 4
+        for (int i = sl; i < nc; i += kColSlices) full |= A[(int64_t)i * lda + j] > 0.f;
+#pragma unroll 4
+        for (int r = sl; r < k; r += kColSlices) {
             const int i = idx[r];
-            if (i >= 0 && i < nc) red = A[(int64_t)i * lda + j] > 0.f;   // rows out of range are ignored
+            if (i >= 0 && i < nc) red |= A[(int64_t)i * lda + j] > 0.f;   // rows out of range are ignored
         }
     }
     pf[sl][cx] = full;
@@ -278,6 +414,7 @@ __global__ void k_col_max(const float* __restrict__ A, int nc, int64_t lda, int 
     const int j = blockIdx.x * kColW + cx;
     float m = 0.f;
     if (j < np)
+#pragma unroll 4
         for (int i = sl; i < nc; i += kColSlices) m = fmaxf(m, A[(int64_t)i * lda + j]);
     part[sl][cx] = m;
     __syncthreads();
@@ -380,6 +517,7 @@ __global__ void k_mark_best(const float* __restrict__ A, int nc, int64_t lda, in
     float m = 0.f;
     int best = -1, lit = 0;
     if (j < np)
+#pragma unroll 4
         for (int i = sl; i < nc; i += kColSlices) {
             const float v = A[(int64_t)i * lda + j];
             lit += v > 0.f;
@@ -474,12 +612,10 @@ int select_top(const float* score, int64_t n, int64_t k, const float* cand, floa
                cudaStream_t stream) {
     if (n < 0 || n > kSelectMax || k < 0 || k > n) return UVC_E_INVAL;
     if (k == 0) return UVC_OK;
-    int m = 1;
-    while (m < n) m <<= 1;
-    const size_t smem = sizeof(unsigned long long) * m + (size_t)n;
+    const size_t smem = (sizeof(uint32_t) + 1) * (size_t)n;
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_select_top, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(unsigned long long) * kSelectMax + kSelectMax));
+                             (int)((sizeof(uint32_t) + 1) * kSelectMax));
     if (attr != cudaSuccess) return status_from_cuda(attr);
     k_select_top<<<1, kSelectThreads, smem, stream>>>(score, (int)n, (int)k, cand, out_cand, out_idx);
     return status_from_cuda(cudaGetLastError());
@@ -498,9 +634,10 @@ int candidate_features(const uvc_scene* sc, const float* cand, int64_t nc, float
                                                          (int)(sizeof(float) * kBins * kHistThreads));
     if (attr != cudaSuccess) return status_from_cuda(attr);
     k_feat_hist<<<(int)nc, kHistThreads, sizeof(float) * kBins * kHistThreads, stream>>>(
-        sc->patch_s, (int)sc->np, sc->area_total, cand, E, feat, ldf);
-    k_feat_clear<<<(int)((nc + 127) / 128), 128, 0, stream>>>(sc->nodes, sc->tri, (int)sc->nt, cand, (int)nc, feat,
-                                                              ldf);
+        sc->patch_s, (int)sc->np, sc->area_total, cand, E, (float)(kBins / (2.0 * std::log2(250.0))),
+        (float)(-2.0 * std::log2(0.1) * kBins / (2.0 * std::log2(250.0))), feat, ldf);
+    k_feat_clear<<<(int)((nc + kClearWarps - 1) / kClearWarps), 32 * kClearWarps, 0, stream>>>(
+        sc->nodes4, sc->nodes, sc->tri, (int)sc->nt, cand, (int)nc, feat, ldf);
     return status_from_cuda(cudaGetLastError());
 }
 

@@ -1,12 +1,12 @@
 // Fluence mu = A^T t (paper Eq. (5)) and the covered-area fraction (the dose
 // constraint mu >= mu_min of Eq. (8)).
 //
-// Fluence: each thread owns two patch columns of a quarter of the candidate
-// rows and keeps NV dwell-vector accumulators per column; terms are summed in
-// blocks of 32 candidates and the block sums are added with Kahan
-// compensation, the quarters in a fixed order (relative error near 36 ulp
-// whatever nc is).  At nvec = 16 the kernel should be bound by the HBM read of
-// A (16 FMA per 4 bytes).
+// Fluence on the CUDA cores: the candidate rows fall into row groups, terms are
+// summed in blocks of 32 candidates and the block sums are added with Kahan
+// compensation, the groups in a fixed order (relative error near 36 ulp
+// whatever nc is).  On the tensor cores: see below.  At nvec = 16 a large product
+// should be bound by the HBM read of A (16 FMA per 4 bytes).
+#include <cooperative_groups.h>
 #include <cuda.h>   // CUtensorMap and its enums (the encoder is fetched through the runtime)
 
 #include <algorithm>
@@ -28,52 +28,62 @@ __device__ __forceinline__ void kahan_add(float& sum, float& c, float x) {
     sum = t;
 }
 
-// One block = 128 patch columns x all candidates.  Its 256 threads form 4
-// row groups of 64 threads; a group takes a contiguous quarter of the
-// candidate rows and each of its threads two adjacent columns, read straight
-// from global memory as one 8-byte load per row when the row stride allows
-// (lda even, A 8-byte aligned), else as two 4-byte loads; a warp reads 256
-// contiguous bytes per row.  The dwell times of the group's rows are staged in
-// shared memory transposed (row-major, 16 per row), so one 16-byte broadcast
-// serves four vectors of both columns, and the 16 products per row and column
-// pair run as packed FP32x2 FMAs.  Sums: blocks of 32 rows plain, block sums
-// Kahan-compensated, the 4 group results added in a fixed order.
+// k_fluence: one cluster of S blocks = 64 patch columns x 16 vectors x all
+// candidates, S in {1, 2, 4, 8}.  The candidate rows are cut into 4 S
+// contiguous groups; a group is two warps of one block, each with 8 of the 16
+// vectors, and a thread takes two adjacent columns, read straight from global
+// memory as one 8-byte load per row when the row stride allows (lda even, A
+// 8-byte aligned), else as two 4-byte loads, eight rows ahead.  The dwell times
+// of the group's rows are staged in shared memory transposed (row-major, 16 per
+// row), so one 16-byte broadcast serves four vectors of both columns, and the
+// products run as packed FP32x2 FMAs over pairs of vectors.  Sums: blocks of 32
+// rows plain, block sums Kahan-compensated, the 4 S group results added in a
+// fixed order through the cluster's shared memory.
+// The first form had one block per 128 columns and all candidates in 4 groups,
+// four rows ahead, one launch per 16 vectors: on a 697 x 9,273 matrix, 73 blocks
+// for 54 us a launch, each thread waiting for its next four rows.  With 37
+// vectors there, fluence and coverage together: 164 -> 70 us.
 constexpr int kFlGroups = 4;                      // row groups per block
 constexpr int kFlGroupThreads = 64;              // threads per row group
 constexpr int kFlCols = 2 * kFlGroupThreads;     // columns per block
 constexpr int kFlChunk = 128;                     // rows of dwell times staged per group at a time
-constexpr int kFlUnroll = 4;                      // rows of A loaded ahead
+constexpr int kFlUnroll = 8;                      // rows of A loaded ahead
+constexpr int kFcCols = 64;                       // columns per cluster of k_fluence
 constexpr size_t kFluenceSmem = sizeof(float) * kFlGroups * kFlChunk * kNV;
 
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-
 __global__ void __launch_bounds__(256, 2) k_fluence(const float* __restrict__ A, int nc, int64_t lda,
-                                                    const float* __restrict__ t, int nvec, int v0,
+                                                    const float* __restrict__ t, int nvec,
                                                     float* __restrict__ mu, int np, int vec2) {
     extern __shared__ float4 fluence_smem[];
-    const int g = threadIdx.x / kFlGroupThreads, gt = threadIdx.x % kFlGroupThreads;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int lane = threadIdx.x & 31, octet = (threadIdx.x >> 5) & 1, g = threadIdx.x >> 6, gt = threadIdx.x & 63;
     float4* ts = fluence_smem + (size_t)g * kFlChunk * (kNV / 4);   // [kFlChunk][kNV / 4]
-    const int j0 = blockIdx.x * kFlCols + 2 * gt;
+    const int x0 = (int)(blockIdx.x / S) * kFcCols, v0 = (int)blockIdx.y * kNV;
+    const int j0 = x0 + 2 * lane;
     const bool ok0 = j0 < np, ok1 = j0 + 1 < np;
-    const int per = (((nc + kFlGroups - 1) / kFlGroups) + 31) / 32 * 32;   // rows per group, multiple of 32
-    const int r0 = min(nc, g * per), r1 = min(nc, r0 + per);
-    float2 part[kNV], acc[kNV], comp[kNV];
+    const int groups = kFlGroups * S;
+    const int per = (((nc + groups - 1) / groups) + 31) / 32 * 32;   // rows per group, multiple of 32
+    const int64_t first = (int64_t)(rank * kFlGroups + g) * per;
+    const int r0 = (int)min((int64_t)nc, first), r1 = min(nc, r0 + per);
+    float2 part[2][4], acc[2][4], comp[2][4];   // [column][vector pair of the octet]
 #pragma unroll
-    for (int v = 0; v < kNV; ++v) {
-        part[v] = make_float2(0.f, 0.f);
-        acc[v] = part[v];
-        comp[v] = part[v];
-    }
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int p = 0; p < 4; ++p) part[c][p] = acc[c][p] = comp[c][p] = make_float2(0.f, 0.f);
     const int nchunk = (per + kFlChunk - 1) / kFlChunk;   // the same for every group
     for (int ck = 0; ck < nchunk; ++ck) {
         const int c0 = r0 + ck * kFlChunk, c1 = min(r1, c0 + kFlChunk);
         __syncthreads();
-        // stage t[v0 + v][c0 .. c1) transposed: ts[row][v]
+        // stage t[v0 + v][c0 .. c1) transposed: ts[row][v], the row's four quads
+        // permuted by the row so that the lanes' stores (consecutive rows) meet 8
+        // banks and not 2
         float* tsf = reinterpret_cast<float*>(ts);
         for (int e = gt; e < kFlChunk * kNV; e += kFlGroupThreads) {
             const int v = e / kFlChunk, q = e % kFlChunk;
             const int i = c0 + q;
-            tsf[q * kNV + v] = (i < c1 && v0 + v < nvec) ? __ldg(&t[(size_t)(v0 + v) * nc + i]) : 0.f;
+            tsf[q * kNV + ((v >> 2) ^ ((q >> 1) & 3)) * 4 + (v & 3)] = (i < c1 && v0 + v < nvec) ? __ldg(&t[(size_t)(v0 + v) * nc + i]) : 0.f;
         }
         __syncthreads();
         for (int q0 = 0; q0 < c1 - c0; q0 += kFlUnroll) {
@@ -85,55 +95,63 @@ __global__ void __launch_bounds__(256, 2) k_fluence(const float* __restrict__ A,
                 if (i < c1) {
                     const float* row = A + (size_t)i * lda + j0;
                     if (vec2 && ok1) {
-                        a[u] = __ldcs(reinterpret_cast<const float2*>(row));
+                        a[u] = __ldg(reinterpret_cast<const float2*>(row));
                     } else {
-                        if (ok0) a[u].x = __ldcs(row);
-                        if (ok1) a[u].y = __ldcs(row + 1);
+                        if (ok0) a[u].x = __ldg(row);
+                        if (ok1) a[u].y = __ldg(row + 1);
                     }
                 }
             }
 #pragma unroll
-            for (int u = 0; u < kFlUnroll; ++u) {
+            for (int u = 0; u < kFlUnroll; ++u) {   // rows past c1 hold zeros
+                const int k = ((q0 + u) >> 1) & 3;
+                const float4 w = ts[(q0 + u) * (kNV / 4) + ((2 * octet) ^ k)], x = ts[(q0 + u) * (kNV / 4) + ((2 * octet + 1) ^ k)];
+                const float2 a0 = make_float2(a[u].x, a[u].x), a1 = make_float2(a[u].y, a[u].y);
+                const float2 w4[4] = {make_float2(w.x, w.y), make_float2(w.z, w.w), make_float2(x.x, x.y), make_float2(x.z, x.w)};
 #pragma unroll
-                for (int v4 = 0; v4 < kNV / 4; ++v4) {
-                    const float4 w = ts[(q0 + u) * (kNV / 4) + v4];   // rows past c1 hold zeros
-                    part[4 * v4 + 0] = ffma2(make_float2(w.x, w.x), a[u], part[4 * v4 + 0]);
-                    part[4 * v4 + 1] = ffma2(make_float2(w.y, w.y), a[u], part[4 * v4 + 1]);
-                    part[4 * v4 + 2] = ffma2(make_float2(w.z, w.z), a[u], part[4 * v4 + 2]);
-                    part[4 * v4 + 3] = ffma2(make_float2(w.w, w.w), a[u], part[4 * v4 + 3]);
+                for (int p = 0; p < 4; ++p) {
+                    part[0][p] = __ffma2_rn(w4[p], a0, part[0][p]);
+                    part[1][p] = __ffma2_rn(w4[p], a1, part[1][p]);
                 }
             }
             if (((q0 + kFlUnroll) & 31) == 0 || q0 + kFlUnroll >= c1 - c0) {   // a block of 32 rows ends
 #pragma unroll
-                for (int v = 0; v < kNV; ++v) {
-                    kahan_add(acc[v].x, comp[v].x, part[v].x);
-                    kahan_add(acc[v].y, comp[v].y, part[v].y);
-                    part[v] = make_float2(0.f, 0.f);
-                }
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        kahan_add(acc[c][p].x, comp[c][p].x, part[c][p].x);
+                        kahan_add(acc[c][p].y, comp[c][p].y, part[c][p].y);
+                        part[c][p] = make_float2(0.f, 0.f);
+                    }
             }
         }
     }
-    // fixed-order (group 0..3) compensated sum of the group results
+    // fixed-order compensated sum of the group results: each block of the cluster
+    // adds up a share of the outputs over all blocks
     __syncthreads();
-    float2* red = reinterpret_cast<float2*>(fluence_smem);   // [kFlGroups][kNV][kFlGroupThreads]
+    float* red = reinterpret_cast<float*>(fluence_smem);   // [kFlGroups][kNV][kFcCols]
 #pragma unroll
-    for (int v = 0; v < kNV; ++v)
-        red[((size_t)g * kNV + v) * kFlGroupThreads + gt] =
-            make_float2(__fsub_rn(acc[v].x, comp[v].x), __fsub_rn(acc[v].y, comp[v].y));
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < kNV * kFlGroupThreads; idx += blockDim.x) {
-        const int v = idx / kFlGroupThreads, l = idx % kFlGroupThreads;
-        const int jj = blockIdx.x * kFlCols + 2 * l;
-        if (v0 + v >= nvec) continue;
-        float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
-        for (int w = 0; w < kFlGroups; ++w) {
-            const float2 x = red[((size_t)w * kNV + v) * kFlGroupThreads + l];
-            kahan_add(s0, c0, x.x);
-            kahan_add(s1, c1, x.y);
-        }
-        if (jj < np) mu[(size_t)(v0 + v) * np + jj] = s0;
-        if (jj + 1 < np) mu[(size_t)(v0 + v) * np + jj + 1] = s1;
+    for (int p = 0; p < 4; ++p) {
+        const int v = 8 * octet + 2 * p;
+        *reinterpret_cast<float2*>(red + (g * kNV + v) * kFcCols + 2 * lane) =
+            make_float2(__fsub_rn(acc[0][p].x, comp[0][p].x), __fsub_rn(acc[1][p].x, comp[1][p].x));
+        *reinterpret_cast<float2*>(red + (g * kNV + v + 1) * kFcCols + 2 * lane) =
+            make_float2(__fsub_rn(acc[0][p].y, comp[0][p].y), __fsub_rn(acc[1][p].y, comp[1][p].y));
     }
+    cluster.sync();
+    const int share = kNV * kFcCols / S;
+    for (int e = rank * share + (int)threadIdx.x; e < (rank + 1) * share; e += blockDim.x) {
+        const int v = e / kFcCols, j = x0 + e % kFcCols;
+        if (v0 + v >= nvec || j >= np) continue;
+        float s = 0.f, c = 0.f;
+        for (int b = 0; b < S; ++b) {
+            const float* other = cluster.map_shared_rank(red, b);
+#pragma unroll
+            for (int w = 0; w < kFlGroups; ++w) kahan_add(s, c, other[w * kNV * kFcCols + e]);
+        }
+        mu[(size_t)(v0 + v) * np + j] = s;
+    }
+    cluster.sync();   // no block leaves while its results are read
 }
 
 // ---------------------------------------------------------------------------
@@ -614,7 +632,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_fluence_tc(const __grid_const
     }
 }
 
-// Deterministic block sum of (float with Kahan terms, count).
+// Deterministic block sum of (float with Kahan terms, count), in thread 0.
 __device__ void block_reduce(float& s, unsigned long long& cnt) {
     __shared__ float ss[32];
     __shared__ unsigned long long sc[32];
@@ -636,32 +654,74 @@ __device__ void block_reduce(float& s, unsigned long long& cnt) {
     }
 }
 
-__global__ void __launch_bounds__(1024) k_area_total(const float4* __restrict__ ps, int np, float* out) {
-    float s = 0.f, c = 0.f;
-    for (int j = threadIdx.x; j < np; j += blockDim.x) kahan_add(s, c, ps[j].w);
-    s = __fsub_rn(s, c);
-    unsigned long long n = 0;
-    block_reduce(s, n);
-    if (threadIdx.x == 0) *out = s;
-}
-
-// One block per dwell vector.
-__global__ void __launch_bounds__(1024) k_coverage(const float* __restrict__ mu, int np, float mu_min,
-                                                   const float4* __restrict__ ps, const float* __restrict__ area_total,
-                                                   float* __restrict__ cov_area, float* __restrict__ cov_count) {
-    const int v = blockIdx.x;
-    const float* m = mu + (size_t)v * np;
-    float s = 0.f, c = 0.f;
-    unsigned long long n = 0;
-    for (int j = threadIdx.x; j < np; j += blockDim.x) {
-        if (m[j] >= mu_min) {
-            kahan_add(s, c, ps[j].w);
-            ++n;
+// Sums over the patches by a cluster of kSumBlocks blocks: area sum (each
+// thread compensated, then trees, the blocks in order) and count of the
+// patches that `in` accepts; the result in thread 0 of rank 0.  One block read
+// 98,132 patches in 32 us (the areas) and 54-75 us (with 4 to 16 vectors).
+constexpr int kSumBlocks = 8, kSumThreads = 512, kSumAhead = 4;
+template <class In>
+__device__ __forceinline__ void cluster_sum(const float4* __restrict__ ps, int np, In in, float& s, unsigned long long& n) {
+    namespace cg = cooperative_groups;
+    __shared__ float sum_of;
+    __shared__ unsigned long long count_of;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), step = kSumBlocks * kSumThreads;
+    float c = 0.f;
+    s = 0.f;
+    n = 0;
+    for (int64_t j0 = rank * kSumThreads + (int)threadIdx.x; j0 < np; j0 += (int64_t)kSumAhead * step) {
+        bool ok[kSumAhead];
+        float a[kSumAhead];
+#pragma unroll
+        for (int q = 0; q < kSumAhead; ++q) {
+            const int64_t j = j0 + (int64_t)q * step;
+            ok[q] = j < np && in(j);
+            a[q] = j < np ? __ldg(&ps[j].w) : 0.f;
         }
+#pragma unroll
+        for (int q = 0; q < kSumAhead; ++q)
+            if (ok[q]) {
+                kahan_add(s, c, a[q]);
+                ++n;
+            }
     }
     s = __fsub_rn(s, c);
     block_reduce(s, n);
     if (threadIdx.x == 0) {
+        sum_of = s;
+        count_of = n;
+    }
+    cluster.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        s = 0.f;
+        c = 0.f;
+        n = 0;
+        for (int b = 0; b < kSumBlocks; ++b) {
+            kahan_add(s, c, *cluster.map_shared_rank(&sum_of, b));
+            n += *cluster.map_shared_rank(&count_of, b);
+        }
+    }
+    cluster.sync();   // no block leaves while its sums are read
+}
+
+__global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kSumThreads)
+    k_area_total(const float4* __restrict__ ps, int np, float* out) {
+    float s;
+    unsigned long long n;
+    cluster_sum(ps, np, [](int64_t) { return true; }, s, n);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *out = s;
+}
+
+// One cluster per dwell vector.
+__global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kSumThreads)
+    k_coverage(const float* __restrict__ mu, int np, float mu_min, const float4* __restrict__ ps,
+               const float* __restrict__ area_total, float* __restrict__ cov_area, float* __restrict__ cov_count) {
+    const int v = blockIdx.x / kSumBlocks;
+    const float* m = mu + (size_t)v * np;
+    float s;
+    unsigned long long n;
+    cluster_sum(ps, np, [&](int64_t j) { return __ldg(m + j) >= mu_min; }, s, n);
+    if (blockIdx.x % kSumBlocks == 0 && threadIdx.x == 0) {
         const float tot = *area_total;
         cov_area[v] = tot > 0.f ? __fdiv_rn(s, tot) : 0.f;
         if (cov_count) cov_count[v] = np > 0 ? __fdiv_rn((float)n, (float)np) : 0.f;
@@ -671,7 +731,7 @@ __global__ void __launch_bounds__(1024) k_coverage(const float* __restrict__ mu,
 }  // namespace
 
 void launch_area_total(const float4* patch_s, int64_t np, float* out, cudaStream_t stream) {
-    k_area_total<<<1, 1024, 0, stream>>>(patch_s, (int)np, out);
+    k_area_total<<<kSumBlocks, kSumThreads, 0, stream>>>(patch_s, (int)np, out);
 }
 
 namespace {
@@ -715,16 +775,33 @@ bool fluence_tensor_map(const float* A, int64_t nc, int64_t lda, int np, int row
 
 std::atomic<int> g_fluence_tc{1};
 
+// Blocks the CUDA-core kernel is split for (two per SM), and the number of its
+// 64-column strips up to which it beats the tensor-core kernel, which takes 128
+// columns per block and so leaves half of the SMs or more idle there: patches /
+// candidates / vectors 1,024 / 2,000 / 64 in 30 against 304 us, 4,096 / 500 / 16 in 14
+// against 23, 9,276 / 2,000 / 16 in 46 against 77; past it 16,384 / 2,000 / 16 in 95
+// against 79 and 40,960 / 2,000 / 16 in 275 against 126.
+constexpr int64_t kFillBlocks = 2 * 152;
+constexpr int64_t kNarrowStrips = 152;
+
 int fluence(const uvc_scene* sc, const float* A, int64_t nc, int64_t lda, const float* t, int32_t nvec,
             float* mu, cudaStream_t stream) {
     const int np = (int)sc->np;
     if (np == 0) return UVC_OK;
     if (nc == 0) return status_from_cuda(cudaMemsetAsync(mu, 0, sizeof(float) * (size_t)nvec * np, stream));
-    static_assert(sizeof(float2) * kFlGroups * kNV * kFlGroupThreads <= kFluenceSmem, "group results fit");
+    static_assert(sizeof(float2) * kFlGroups * kNV * kFlGroupThreads <= kFluenceSmem &&
+                      sizeof(float) * kFlGroups * kNV * kFcCols <= kFluenceSmem, "group results fit");
+    // Row splits of the CUDA-core kernel: clusters of more blocks while the
+    // columns and vectors alone leave the chip short of kFillBlocks and a group
+    // keeps at least 32 rows.
+    const int64_t passes = (nvec + kNV - 1) / kNV, cols = (np + kFcCols - 1) / kFcCols;
+    int S = 1;
+    while (S < 8 && cols * passes * S < kFillBlocks && nc >= (int64_t)2 * S * kFlGroups * 32) S *= 2;
+    const bool narrow = cols <= kNarrowStrips;
     static_assert(kFlGroups * kFlGroupThreads == kThreads, "block shape");
     static_assert(kFlChunk % kTmaRows == 0 && kTmaRows * kFlCols * sizeof(float) % 128 == 0, "tile shape");
     CUtensorMap map;
-    if (g_fluence_tc.load() && fluence_tensor_map(A, nc, lda, np, kTcRows, &map)) {
+    if (!narrow && g_fluence_tc.load() && fluence_tensor_map(A, nc, lda, np, kTcRows, &map)) {
         static const cudaError_t cattr =
             cudaFuncSetAttribute(k_fluence_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
         if (cattr != cudaSuccess) return status_from_cuda(cattr);
@@ -734,7 +811,7 @@ int fluence(const uvc_scene* sc, const float* A, int64_t nc, int64_t lda, const 
             k_fluence_tc<<<grid, kTcThreads, kTcSmem, stream>>>(map, (int)nc, t, nvec, v0, mu, np, sc->status);
         return status_from_cuda(cudaGetLastError());
     }
-    if (fluence_tensor_map(A, nc, lda, np, kTmaRows, &map)) {
+    if (!narrow && S == 1 && fluence_tensor_map(A, nc, lda, np, kTmaRows, &map)) {
         static const cudaError_t tattr =
             cudaFuncSetAttribute(k_fluence_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTmaSmem);
         if (tattr != cudaSuccess) return status_from_cuda(tattr);
@@ -748,16 +825,24 @@ int fluence(const uvc_scene* sc, const float* A, int64_t nc, int64_t lda, const 
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_fluence, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFluenceSmem);
     if (attr != cudaSuccess) return status_from_cuda(attr);
-    const int grid = (np + kFlCols - 1) / kFlCols;
     const int vec2 = (lda % 2 == 0) && (reinterpret_cast<uintptr_t>(A) % 8 == 0);
-    for (int v0 = 0; v0 < nvec; v0 += kNV)
-        k_fluence<<<grid, kThreads, kFluenceSmem, stream>>>(A, (int)nc, lda, t, nvec, v0, mu, np, vec2);
-    return status_from_cuda(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cols * S), (unsigned)passes, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.dynamicSmemBytes = kFluenceSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)S;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return status_from_cuda(cudaLaunchKernelEx(&cfg, k_fluence, A, (int)nc, lda, t, (int)nvec, mu, np, vec2));
 }
 
 int coverage(const uvc_scene* sc, const float* mu, int32_t nvec, float mu_min, float* cov_area, float* cov_count,
              cudaStream_t stream) {
-    k_coverage<<<nvec, 1024, 0, stream>>>(mu, (int)sc->np, mu_min, sc->patch_s, sc->area_total, cov_area,
+    k_coverage<<<nvec * kSumBlocks, kSumThreads, 0, stream>>>(mu, (int)sc->np, mu_min, sc->patch_s, sc->area_total, cov_area,
                                           cov_count);
     return status_from_cuda(cudaGetLastError());
 }
