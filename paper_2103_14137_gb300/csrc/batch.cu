@@ -52,7 +52,7 @@ static_assert(sizeof(LampPack) + 64 <= 32764, "kernel parameters");
 // lamp of the batch takes the wedge path, 1 = all do, 2 = mixed (chosen per
 // job; both paths inlined).  PACK: the lamps and jobs come from `pack`.
 template <int MODE, bool PACK>
-__global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
+__global__ void __launch_bounds__(kThreads, kCallMinBlocks)
     k_irradiance_batch(const JobDev* __restrict__ jobs, int njobs, const LampDev* __restrict__ lamps,
                        const __grid_constant__ LampPack pack, int cpt, int64_t task_lo, int64_t task_hi,
                        int stack_cap, int wedge_k) {
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
         const LampDev& L = PACK ? pack.L[J.lamp] : lamps[J.lamp];
         for (int i = ic * cpt; i < i1; ++i) {
             const bool wedge = MODE == 1 || (MODE == 2 && L.wedge);
-            const float E = wedge ? irradiance_wedge<false>(J.S, J.cand, J.nc, L, i, jb, lane, stack, ws, J.vis,
+            const float E = wedge ? irradiance_wedge<false, true, true>(J.S, J.cand, J.nc, L, i, jb, lane, stack, ws, J.vis,
                                                             J.njb, P, cache)
                                   : irradiance_entry<false>(J.S, J.cand, J.nc, L, i, jb, lane, stack, J.vis,
                                                             J.njb, P, cache);

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS) k_irradiance(Sce
         const int i1 = min(nc, (ic + 1) * kCandPerTask);
         for (int i = ic * kCandPerTask; i < i1; ++i) {
             const float E =
-                WEDGE ? irradiance_wedge<COUNT>(S, cand, nc, L, i, jb, lane, stack, ws, vis, njb, P, cache, ctr)
+                WEDGE ? irradiance_wedge<COUNT, !COUNT>(S, cand, nc, L, i, jb, lane, stack, ws, vis, njb, P, cache, ctr)
                       : irradiance_entry<COUNT>(S, cand, nc, L, i, jb, lane, stack, vis, njb, P, cache, ctr);
             if (P.valid) A[(size_t)i * lda + j] = E;
         }

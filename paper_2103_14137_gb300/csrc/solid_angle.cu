@@ -186,8 +186,8 @@ __device__ __forceinline__ uint32_t packet_to(const SceneView& S, float ox, floa
 // traversal in traverse.cuh); the per-source results, and so the entries, are
 // those of the source-by-source searches.
 template <bool WEDGE>
-__global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
-    k_area_mean(SceneView S, const float* __restrict__ cand, int nc, LampDev L, const float* __restrict__ ptri,
+__global__ void __launch_bounds__(kThreads, kCallMinBlocks)
+    k_area_mean(const __grid_constant__ SceneView S, const float* __restrict__ cand, int nc, const __grid_constant__ LampDev L, const float* __restrict__ ptri,
                 float* __restrict__ A, int64_t lda, uint8_t* __restrict__ nclosed, const int2* __restrict__ tri_place, int cpt) {
     extern __shared__ __align__(16) int smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
             if (WEDGE) {
                 uint32_t want;
                 float lend, dmax, gx, gy, sum;
-                const uint32_t facing = wedge_setup_patch(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, sum);
+                const uint32_t facing = wedge_setup_patch<false>(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, sum);
                 uint32_t vis_c = 0u, all = 0u;   // all: sources that saw every check point so far
                 // q = -1: the centroid; q = 0..5: the check points.  One call site of
                 // the (large, inlined) wedge search keeps the kernel's code small.
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS)
                         if (!(plq.gap > 0.f)) plq.own_axis = -1;
                     }
                     uint32_t fq;
-                    const uint32_t oc = wedge_search<false>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex, plq, lane, stack, ws, cache, fq, nullptr);
+                    const uint32_t oc = wedge_search<false, true>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex, plq, lane, stack, ws, cache, fq, nullptr);
                     failed_all |= fq;
                     if (q < 0) {
                         vis_c = ((fq >> lane) & 1u) ? 0u : (facing & ~oc);

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "uvc_internal.cuh"
 
@@ -846,6 +847,8 @@ struct WedgeSmem {
     uint32_t* qitem;          // [kLeafQueue]: lane << 27 | leaf
     uint32_t* occ;            // [32]
     int* qhit;                // [32]
+    char* base;               // where the arrays of all the block's warps start, and the K they are laid out for
+    int base_k;
 };
 
 // Shared memory of a block of the traversal kernels: the warps' stacks
@@ -861,6 +864,8 @@ inline size_t wedge_smem_bytes(int K) {
 
 __device__ __forceinline__ WedgeSmem wedge_smem(char* base, int K, int warp) {
     WedgeSmem w;
+    w.base = base;
+    w.base_k = K;
     const size_t per_src = (size_t)kWarpsPerBlock * K * 32;
     w.shear = reinterpret_cast<float4*>(base) + (size_t)warp * K * 32;
     w.term = reinterpret_cast<float*>(base + per_src * sizeof(float4)) + (size_t)warp * K * 32;
@@ -1082,6 +1087,10 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b, float2 m1) { return _
 // sources and, in `want`, those that need a search (facing, longer than the
 // clearance cut), with the largest cut parameter `lend`, the longest such
 // segment `dmax` and the common horizontal direction (gx, gy).
+// MODES: separate passes for horizontal and vertical normals (the walls, floors
+// and ceilings of rooms: ward matrix 8.6 -> 8.1 ms).  They cost registers that
+// the streamed kernel does not have (3.9 -> 5.4 ms there).
+template <bool MODES>
 __device__ __forceinline__ uint32_t wedge_setup_patch(const SceneView& S, const LampDev& L, float cx, float cy,
                                                       float cz, const PatchLane& P, int lane, const WedgeSmem& ws,
                                                       uint32_t& want, float& lend, float& dmax, float& gx,
@@ -1110,34 +1119,55 @@ __device__ __forceinline__ uint32_t wedge_setup_patch(const SceneView& S, const 
     uint32_t facing = 0;
     float far2 = 0.f;
     sum = 0.f;
-    for (int m = 0; m < L.K; m += 2) {
-        const int k = min(m + 1, L.K - 1);   // an odd lamp's last source twice; its second half is dropped
-        const float2 oz = __fadd2_rn(c2, make_float2(L.oz[m], L.oz[k]));
-        const float2 hz = sub2(oz, sz, m1), qz = sub2(hz, oz, m1);
-        const float2 lz = __fadd2_rn(sub2(oz, sub2(hz, qz, m1), m1), sub2(szn, qz, m1));
-        const float2 pn = __fmul2_rn(nzn, hz), e3 = __ffma2_rn(nz, hz, pn);   // pn = -(n.z h.z)
-        const float2 s = sub2(acc, pn, m1), z = sub2(s, acc, m1);
-        const float2 q = sub2(sub2(acc, sub2(s, z, m1), m1), __fadd2_rn(pn, z), m1);
-        const float2 nv = __fadd2_rn(s, __ffma2_rn(nz, lz, __fadd2_rn(err, __fadd2_rn(q, e3))));
-        const float2 d2 = __ffma2_rn(hx2, hx2, __ffma2_rn(hy2, hy2, __fmul2_rn(hz, hz)));
-        const float2 r = make_float2(rsqrt_approx(d2.x), rsqrt_approx(d2.y));
-        const float2 r2 = __fmul2_rn(r, r), r3 = __fmul2_rn(r2, r), f = __ffma2_rn(d2, r2, m1);
-        const float2 w = __ffma2_rn(__fmul2_rn(f, make_float2(-1.5f, -1.5f)), r3, r3);
-        float2 t = __fmul2_rn(make_float2(L.pw[m], L.pw[k]), __fmul2_rn(nv, w));
-        bool f0 = nv.x > 0.f, f1 = nv.y > 0.f && k > m;
-        if (!(fminf(d2.x, d2.y) >= kTermMin && fmaxf(d2.x, d2.y) <= kTermMax)) {
-            f0 = f0 && d2.x > 0.f;
-            f1 = f1 && d2.y > 0.f;
-            t = make_float2(source_term(L.pw[m], nv.x, d2.x), source_term(L.pw[k], nv.y, d2.y));
+    // One pass over the pairs of sources.  NORMAL: 0 = any normal; 1 = horizontal
+    // normals (n.z = 0), where <n, v> is the same for all sources; 2 = vertical
+    // ones, where it is n.z times the rounded height difference (the rounded sum
+    // of a rounded difference and its error is that difference).  Each gives what
+    // the general form does.
+    auto pass = [&](auto normal) {
+        constexpr int NORMAL = decltype(normal)::value;
+        const float nv0 = __fadd_rn(acc0, err0);
+        for (int m = 0; m < L.K; m += 2) {
+            const int k = min(m + 1, L.K - 1);   // an odd lamp's last source twice; its second half is dropped
+            const float2 oz = __fadd2_rn(c2, make_float2(L.oz[m], L.oz[k]));
+            const float2 hz = sub2(oz, sz, m1);
+            float2 nv;
+            if constexpr (NORMAL == 1) {
+                nv = dup2(nv0);
+            } else if constexpr (NORMAL == 2) {
+                nv = __fmul2_rn(nz, hz);
+            } else {
+                const float2 qz = sub2(hz, oz, m1);
+                const float2 lz = __fadd2_rn(sub2(oz, sub2(hz, qz, m1), m1), sub2(szn, qz, m1));
+                const float2 pn = __fmul2_rn(nzn, hz), e3 = __ffma2_rn(nz, hz, pn);   // pn = -(n.z h.z)
+                const float2 s = sub2(acc, pn, m1), z = sub2(s, acc, m1);
+                const float2 q = sub2(sub2(acc, sub2(s, z, m1), m1), __fadd2_rn(pn, z), m1);
+                nv = __fadd2_rn(s, __ffma2_rn(nz, lz, __fadd2_rn(err, __fadd2_rn(q, e3))));
+            }
+            const float2 d2 = __ffma2_rn(hx2, hx2, __ffma2_rn(hy2, hy2, __fmul2_rn(hz, hz)));
+            const float2 r = make_float2(rsqrt_approx(d2.x), rsqrt_approx(d2.y));
+            const float2 r2 = __fmul2_rn(r, r), r3 = __fmul2_rn(r2, r), f = __ffma2_rn(d2, r2, m1);
+            const float2 w = __ffma2_rn(__fmul2_rn(f, make_float2(-1.5f, -1.5f)), r3, r3);
+            float2 t = __fmul2_rn(make_float2(L.pw[m], L.pw[k]), __fmul2_rn(nv, w));
+            bool f0 = nv.x > 0.f, f1 = nv.y > 0.f && k > m;
+            if (!(fminf(d2.x, d2.y) >= kTermMin && fmaxf(d2.x, d2.y) <= kTermMax)) {
+                f0 = f0 && d2.x > 0.f;
+                f1 = f1 && d2.y > 0.f;
+                t = make_float2(source_term(L.pw[m], nv.x, d2.x), source_term(L.pw[k], nv.y, d2.y));
+            }
+            t.x = f0 ? t.x : 0.f;
+            t.y = f1 ? t.y : 0.f;
+            ws.term[m * 32 + lane] = t.x;
+            if (k > m) ws.term[k * 32 + lane] = t.y;
+            sum = __fadd_rn(__fadd_rn(sum, t.x), t.y);
+            far2 = fmaxf(far2, fmaxf(f0 ? d2.x : 0.f, f1 ? d2.y : 0.f));
+            facing |= ((uint32_t)f0 << m) | ((uint32_t)f1 << k);
         }
-        t.x = f0 ? t.x : 0.f;
-        t.y = f1 ? t.y : 0.f;
-        ws.term[m * 32 + lane] = t.x;
-        if (k > m) ws.term[k * 32 + lane] = t.y;
-        sum = __fadd_rn(__fadd_rn(sum, t.x), t.y);
-        far2 = fmaxf(far2, fmaxf(f0 ? d2.x : 0.f, f1 ? d2.y : 0.f));
-        facing |= ((uint32_t)f0 << m) | ((uint32_t)f1 << k);
-    }
+    };
+    const bool hor = n4.z == 0.f, ver = n4.x == 0.f && n4.y == 0.f && fabsf(n4.z) == 1.f;
+    if (MODES && __all_sync(kFull, hor || !P.valid)) pass(std::integral_constant<int, 1>());
+    else if (MODES && __all_sync(kFull, ver || !P.valid)) pass(std::integral_constant<int, 2>());
+    else pass(std::integral_constant<int, 0>());
     if (!P.valid) facing = 0u;
     gx = -hx;
     gy = -hy;
@@ -1190,40 +1220,19 @@ __device__ __forceinline__ void wedge_shear(const LampDev& L, float cz, float sz
     }
 }
 
-// The search from the lamp line of candidate c to the lane's point (height sz,
-// horizontal direction (gx, gy) from c) for the sources in `want`: the plates
-// first, then one wedge search of the subtrees with loose triangles for the
-// sources that no plate blocks or leaves open, and one of the whole tree for
-// the open ones (for all where plates are not used).  A wedge search tests the
-// lane's cached occluder, then walks the tree.  Returns the sources found
-// occluded; `failed` gets the lanes whose search hit the visit cap or the
-// stack limit.
+// What the plates leave of a search: one wedge search of the subtrees with
+// loose triangles for the sources in `want` that are not open, and one of the
+// whole tree for the open ones (for all where plates are not used).  A wedge
+// search tests the lane's cached occluder, then walks the tree.  Returns the
+// sources left unoccluded; `failed` gets the lanes whose search hit the visit
+// cap or the stack limit.
 template <bool COUNT>
-__device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampDev& L, float cx, float cy, float cz,
-                                                 float sz, float gx, float gy, uint32_t want, float lend, float dmax,
-                                                 int2 ex, const PlateLane& pl, int lane, int* stack, const WedgeSmem& ws,
-                                                 int& cache, uint32_t& failed, unsigned long long* ctr) {
-    failed = 0;
-    if (S.nt == 0 || !__any_sync(kFull, want != 0u)) return 0u;
+__device__ __forceinline__ uint32_t wedge_rest(const SceneView& S, const LampDev& L, bool plates, float cx, float cy,
+                                               float cz, float sz, float gx, float gy, uint32_t want, uint32_t open,
+                                               float lend, float dmax, int2 ex, int lane, int* stack,
+                                               const WedgeSmem& ws, const Slabs& sl, int& cache, uint32_t& failed,
+                                               unsigned long long* ctr) {
     const float delta = S.cut_eps;
-    const uint32_t before = want;
-    const bool plates = !COUNT && S.nplate != 0 && L.plates;
-    const Slabs sl = slabs_of(cx, cy, gx, gy, delta);
-    uint32_t open = want;
-    if (plates) {
-        float zlo = __fadd_rn(cz, L.zmin), zhi = __fadd_rn(cz, L.zmax);
-        if (__any_sync(kFull, want != 0u && want != (1u << L.K) - 1u) && want) {
-            zlo = 3.0e38f;
-            zhi = -3.0e38f;
-            for (uint32_t b = want; b; b &= b - 1) {
-                const float oz = __fadd_rn(cz, L.oz[__ffs(b) - 1]);
-                zlo = fminf(zlo, oz);
-                zhi = fmaxf(zhi, oz);
-            }
-        }
-        open = plates_decide(S, [&](int q) { return __fadd_rn(cz, L.oz[q]); }, L.K, cx, cy, sz, gx, gy, zlo, zhi, lend,
-                             dmax, sl, pl, lane, want);
-    }
     for (int whole = plates && (S.nplate & kLooseBit) ? 0 : 1; whole < 2; ++whole) {
         uint32_t set = want & (whole ? open : ~open);
         if (!__any_sync(kFull, set != 0u)) continue;
@@ -1296,13 +1305,81 @@ __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampD
         want &= ~(set0 & ~set);
         if (hit_tri >= 0) cache = hit_tri;
     }
+    return want;
+}
+
+// wedge_rest as a call, for kernels that hold much else in registers (the
+// batch's job records, the area mean's patches and gaps): on a room of plates a
+// packet in a hundred gets there.  Measured with 128 registers (two blocks per SM):
+// batched rooms 3.09 -> 2.71 ms, area mean 4.08 -> 3.56 ms; inlined at two blocks
+// 3.07 and 3.83.  The plain and streamed kernels are faster with it inlined at
+// three blocks (ward matrix 8.1 against 8.6 ms, streamed floor 3.9 against 4.1).
+constexpr int kCallMinBlocks = 2;
+struct WedgeRest {
+    uint32_t want, failed;
+    int cache;
+};
+__device__ __noinline__ WedgeRest wedge_rest_call(const SceneView& S, const LampDev& L, bool plates, float cx, float cy,
+                                                  float cz, float sz, float gx, float gy, uint32_t want, uint32_t open,
+                                                  float lend, float dmax, int ex0, int ex1, int* stack, char* base,
+                                                  int base_k, int cache) {
+    WedgeRest r;
+    r.failed = 0u;
+    r.cache = cache;
+    r.want = wedge_rest<false>(S, L, plates, cx, cy, cz, sz, gx, gy, want, open, lend, dmax, make_int2(ex0, ex1),
+                               threadIdx.x & 31, stack, wedge_smem(base, base_k, threadIdx.x >> 5),
+                               slabs_of(cx, cy, gx, gy, S.cut_eps), r.cache, r.failed, nullptr);
+    return r;
+}
+
+// The search from the lamp line of candidate c to the lane's point (height sz,
+// horizontal direction (gx, gy) from c) for the sources in `want`: the plates
+// first, then the hierarchy for what they leave.  Returns the sources found
+// occluded; `failed` as in wedge_rest.  CALL: wedge_rest is called, not inlined.
+template <bool COUNT, bool CALL>
+__device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampDev& L, float cx, float cy, float cz,
+                                                 float sz, float gx, float gy, uint32_t want, float lend, float dmax,
+                                                 int2 ex, const PlateLane& pl, int lane, int* stack, const WedgeSmem& ws,
+                                                 int& cache, uint32_t& failed, unsigned long long* ctr) {
+    failed = 0;
+    if (S.nt == 0 || !__any_sync(kFull, want != 0u)) return 0u;
+    const uint32_t before = want;
+    const bool plates = !COUNT && S.nplate != 0 && L.plates;
+    const Slabs sl = slabs_of(cx, cy, gx, gy, S.cut_eps);
+    uint32_t open = want;
+    if (plates) {
+        float zlo = __fadd_rn(cz, L.zmin), zhi = __fadd_rn(cz, L.zmax);
+        if (__any_sync(kFull, want != 0u && want != (1u << L.K) - 1u) && want) {
+            zlo = 3.0e38f;
+            zhi = -3.0e38f;
+            for (uint32_t b = want; b; b &= b - 1) {
+                const float oz = __fadd_rn(cz, L.oz[__ffs(b) - 1]);
+                zlo = fminf(zlo, oz);
+                zhi = fmaxf(zhi, oz);
+            }
+        }
+        open = plates_decide(S, [&](int q) { return __fadd_rn(cz, L.oz[q]); }, L.K, cx, cy, sz, gx, gy, zlo, zhi, lend,
+                             dmax, sl, pl, lane, want);
+    }
+    if (CALL) {
+        if (__any_sync(kFull, (want & (!plates || (S.nplate & kLooseBit) ? ~0u : open)) != 0u)) {
+            const WedgeRest r = wedge_rest_call(S, L, plates, cx, cy, cz, sz, gx, gy, want, open, lend, dmax, ex.x, ex.y,
+                                                stack, ws.base, ws.base_k, cache);
+            want = r.want;
+            failed = r.failed;
+            cache = r.cache;
+        }
+    } else {
+        want = wedge_rest<COUNT>(S, L, plates, cx, cy, cz, sz, gx, gy, want, open, lend, dmax, ex, lane, stack, ws, sl,
+                                 cache, failed, ctr);
+    }
     return before & ~want;
 }
 
 // Irradiance of candidate i at this lane's patch for a vertical line lamp
 // (L.wedge): the same entry as irradiance_entry, with one search per candidate
 // instead of one per source.
-template <bool COUNT = false>
+template <bool COUNT = false, bool MODES = false, bool CALL = false>
 __device__ __forceinline__ float irradiance_wedge(const SceneView& S, const float* __restrict__ cand, int nc,
                                                   const LampDev& L, int i, int jb, int lane, int* stack,
                                                   const WedgeSmem& ws, uint32_t* __restrict__ vis, int nwords,
@@ -1312,10 +1389,10 @@ __device__ __forceinline__ float irradiance_wedge(const SceneView& S, const floa
     uint32_t want;
     float lend, dmax, gx, gy;
     float E;
-    const uint32_t facing = wedge_setup_patch(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, E);
+    const uint32_t facing = wedge_setup_patch<MODES>(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, E);
     uint32_t failed;
     const PlateLane pl = !COUNT && S.nplate != 0 ? plate_lane(S, jb, lane, P) : no_plate_lane();
-    const uint32_t occl = wedge_search<COUNT>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, pl, lane,
+    const uint32_t occl = wedge_search<COUNT, CALL>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, pl, lane,
                                               stack, ws, cache, failed, ctr);
     const bool bad = (failed >> lane) & 1u;
     const uint32_t visible = bad ? 0u : (facing & ~occl);
