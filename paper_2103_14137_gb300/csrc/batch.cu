@@ -50,9 +50,10 @@ static_assert(sizeof(LampPack) + 64 <= 32764, "kernel parameters");
 // Lamps with the wedge path (LampDev::wedge) use the per-source shared
 // arrays, sized for the batch's largest such lamp (wedge_k).  MODE: 0 = no
 // lamp of the batch takes the wedge path, 1 = all do, 2 = mixed (chosen per
-// job; both paths inlined).  PACK: the lamps and jobs come from `pack`.
-template <int MODE, bool PACK>
-__global__ void __launch_bounds__(kThreads, kCallMinBlocks)
+// job; both paths inlined).  PACK: the lamps and jobs come from `pack`.  PLATES:
+// some job's scene has plates.
+template <int MODE, bool PACK, bool PLATES>
+__global__ void __launch_bounds__(kThreads, PLATES ? kCallMinBlocks : UVC_IRR_MIN_BLOCKS)
     k_irradiance_batch(const JobDev* __restrict__ jobs, int njobs, const LampDev* __restrict__ lamps,
                        const __grid_constant__ LampPack pack, int cpt, int64_t task_lo, int64_t task_hi,
                        int stack_cap, int wedge_k) {
@@ -78,9 +79,9 @@ __global__ void __launch_bounds__(kThreads, kCallMinBlocks)
         const LampDev& L = PACK ? pack.L[J.lamp] : lamps[J.lamp];
         for (int i = ic * cpt; i < i1; ++i) {
             const bool wedge = MODE == 1 || (MODE == 2 && L.wedge);
-            const float E = wedge ? irradiance_wedge<false, true, true>(J.S, J.cand, J.nc, L, i, jb, lane, stack, ws, J.vis,
+            const float E = wedge ? irradiance_wedge<false, PLATES, PLATES, PLATES>(J.S, J.cand, J.nc, L, i, jb, lane, stack, ws, J.vis,
                                                             J.njb, P, cache)
-                                  : irradiance_entry<false>(J.S, J.cand, J.nc, L, i, jb, lane, stack, J.vis,
+                                  : irradiance_entry<false, PLATES>(J.S, J.cand, J.nc, L, i, jb, lane, stack, J.vis,
                                                             J.njb, P, cache);
             if (P.valid) J.A[(size_t)i * J.lda + j] = E;
         }
@@ -89,12 +90,16 @@ __global__ void __launch_bounds__(kThreads, kCallMinBlocks)
 
 using BatchKernel = void (*)(const JobDev*, int, const LampDev*, const LampPack, int, int64_t, int64_t, int, int);
 
-template <bool PACK>
-BatchKernel kernel_for_pack(int mode) {
-    return mode == 0 ? k_irradiance_batch<0, PACK> : (mode == 1 ? k_irradiance_batch<1, PACK> : k_irradiance_batch<2, PACK>);
+template <bool PACK, bool PLATES>
+BatchKernel kernel_for_mode(int mode) {
+    return mode == 0 ? k_irradiance_batch<0, PACK, PLATES>
+                     : (mode == 1 ? k_irradiance_batch<1, PACK, PLATES> : k_irradiance_batch<2, PACK, PLATES>);
 }
 
-BatchKernel kernel_for(int mode, bool pack) { return pack ? kernel_for_pack<true>(mode) : kernel_for_pack<false>(mode); }
+BatchKernel kernel_for(int mode, bool pack, bool plates) {
+    return pack ? (plates ? kernel_for_mode<true, true>(mode) : kernel_for_mode<true, false>(mode))
+                : (plates ? kernel_for_mode<false, true>(mode) : kernel_for_mode<false, false>(mode));
+}
 
 bool valid_cpt(int c) { return c == 1 || c == 2 || c == 4 || c == 8 || c == 16; }
 
@@ -112,6 +117,7 @@ struct uvc_batch {
     int stack_cap = 1;
     int wedge_k = 0;                      // largest K among the lamps with the wedge path
     int mode = 0;                         // kernel variant: 0 no wedge lamp, 1 all wedge, 2 mixed
+    bool plates = false;                  // some job decides segments at plates
     int64_t total_pairs = 0;
     uvc::LampPack pack{};                 // the lamps and jobs again, for the kernel parameters (small batches)
     int uploaded_cpt = 0;                 // cand_per_task of the uploaded table
@@ -146,7 +152,7 @@ int upload(uvc_batch* b, int cpt, cudaStream_t stream, int64_t* total_tasks) {
 int launch_range(const uvc_batch* b, int cpt, int blocks_per_sm, int64_t lo, int64_t hi, cudaStream_t stream) {
     if (hi <= lo) return UVC_OK;
     const bool pack = b->nlamps <= kParamLamps && b->njobs <= kParamJobs;
-    BatchKernel k = kernel_for(b->mode, pack);
+    BatchKernel k = kernel_for(b->mode, pack, b->plates);
     const size_t smem = stack_smem_bytes(b->stack_cap) + wedge_smem_bytes(b->wedge_k);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -231,6 +237,7 @@ int uvc_batch_create(const uvc_job* jobs, int32_t njobs, const uvc_lamp* lamps, 
         }
         uvc::JobDev& D = b->host_jobs[q];
         D.S = uvc::view_of(J.scene);
+        b->plates |= D.S.nplate != 0 && b->host_lamps[J.lamp].plates;
         D.cand = J.cand;
         D.A = J.A;
         D.vis = J.vis;

@@ -42,7 +42,7 @@ namespace {
 #endif
 constexpr int kCandPerTask = UVC_CAND_PER_TASK;
 
-template <bool COUNT, bool WEDGE>
+template <bool COUNT, bool WEDGE, bool PLATES>
 __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS) k_irradiance(SceneView S, const float* __restrict__ cand, int nc,
                                                          LampDev L, float* __restrict__ A, int64_t lda,
                                                          uint32_t* __restrict__ vis, unsigned long long* ctr) {
@@ -67,8 +67,8 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS) k_irradiance(Sce
         const int i1 = min(nc, (ic + 1) * kCandPerTask);
         for (int i = ic * kCandPerTask; i < i1; ++i) {
             const float E =
-                WEDGE ? irradiance_wedge<COUNT, !COUNT>(S, cand, nc, L, i, jb, lane, stack, ws, vis, njb, P, cache, ctr)
-                      : irradiance_entry<COUNT>(S, cand, nc, L, i, jb, lane, stack, vis, njb, P, cache, ctr);
+                WEDGE ? irradiance_wedge<COUNT, PLATES, !COUNT, false>(S, cand, nc, L, i, jb, lane, stack, ws, vis, njb, P, cache, ctr)
+                      : irradiance_entry<COUNT, PLATES>(S, cand, nc, L, i, jb, lane, stack, vis, njb, P, cache, ctr);
             if (P.valid) A[(size_t)i * lda + j] = E;
         }
         jb += djb;
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS) k_irradiance(Sce
 // zeroed before the launch) as they finish instead of a fixed share each;
 // every task's sums are the same whichever warp takes it.
 constexpr int kStreamedBlock = 20;
-template <bool WEDGE>
+template <bool WEDGE, bool PLATES>
 __global__ void __launch_bounds__(kThreads, UVC_STREAMED_MIN_BLOCKS) k_streamed(SceneView S, const float* __restrict__ cand, int nc,
                                                        LampDev L, const float* __restrict__ t, int nvec,
                                                        float* __restrict__ partial, int nsplit, int chunk,
@@ -119,8 +119,8 @@ __global__ void __launch_bounds__(kThreads, UVC_STREAMED_MIN_BLOCKS) k_streamed(
             const int nb = min(kStreamedBlock, i1 - ib);
             for (int q = 0; q < nb; ++q)
                 Et[q * 32 + lane] =
-                    WEDGE ? irradiance_wedge(S, cand, nc, L, ib + q, jb, lane, stack, ws, nullptr, 0, P, cache)
-                          : irradiance_entry(S, cand, nc, L, ib + q, jb, lane, stack, nullptr, 0, P, cache);
+                    WEDGE ? irradiance_wedge<false, PLATES, false, false>(S, cand, nc, L, ib + q, jb, lane, stack, ws, nullptr, 0, P, cache)
+                          : irradiance_entry<false, PLATES>(S, cand, nc, L, ib + q, jb, lane, stack, nullptr, 0, P, cache);
             __syncwarp();
             if (j < S.np) {
                 for (int v = 0; v < nvec; ++v) {
@@ -172,13 +172,17 @@ size_t streamed_smem(const SceneView& S, const LampDev& lamp) {
            (lamp.wedge ? wedge_smem_bytes(lamp.K) : 0);
 }
 
-const void* streamed_kernel(const LampDev& lamp) {
-    return lamp.wedge ? (const void*)k_streamed<true> : (const void*)k_streamed<false>;
+using StreamedKernel = void (*)(const SceneView, const float*, int, const LampDev, const float*, int, float*, int, int,
+                                unsigned long long*);
+StreamedKernel streamed_kernel(const SceneView& S, const LampDev& lamp) {
+    const bool plates = S.nplate != 0 && lamp.plates;
+    return lamp.wedge ? (plates ? k_streamed<true, true> : k_streamed<true, false>)
+                      : (plates ? k_streamed<false, true> : k_streamed<false, false>);
 }
 
 int streamed_grid(const SceneView& S, const LampDev& lamp, int* grid) {
-    const int rc = allow_smem(streamed_kernel(lamp), streamed_smem(S, lamp));
-    *grid = grid_for(streamed_kernel(lamp), streamed_smem(S, lamp));
+    const int rc = allow_smem((const void*)streamed_kernel(S, lamp), streamed_smem(S, lamp));
+    *grid = grid_for((const void*)streamed_kernel(S, lamp), streamed_smem(S, lamp));
     return rc;
 }
 
@@ -189,12 +193,8 @@ int launch_streamed(int grid, const SceneView& S, const float* cand, int64_t nc,
     cudaError_t e = cudaMemsetAsync(next_task, 0, sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return status_from_cuda(e);
     const size_t smem = streamed_smem(S, lamp);
-    if (lamp.wedge)
-        k_streamed<true><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, t, nvec, partial, (int)nsplit,
-                                                           chunk, next_task);
-    else
-        k_streamed<false><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, t, nvec, partial, (int)nsplit,
-                                                            chunk, next_task);
+    streamed_kernel(S, lamp)<<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, t, nvec, partial, (int)nsplit,
+                                                               chunk, next_task);
     return UVC_OK;
 }
 
@@ -203,17 +203,18 @@ int launch_irradiance(const SceneView& S, const float* cand, int64_t nc, const L
                       uint32_t* vis, unsigned long long* ctr, cudaStream_t stream) {
     const bool wedge = lamp.wedge != 0;
     const size_t smem = stack_smem_bytes(S.stack_cap) + (wedge ? wedge_smem_bytes(lamp.K) : 0);
-    const void* kern = wedge ? (const void*)k_irradiance<COUNT, true> : (const void*)k_irradiance<COUNT, false>;
+    using Kernel = void (*)(const SceneView, const float*, int, const LampDev, float*, int64_t, uint32_t*, unsigned long long*);
+    const bool plates = !COUNT && S.nplate != 0 && lamp.plates;
+    const Kernel kernel = wedge ? (plates ? k_irradiance<COUNT, true, !COUNT> : k_irradiance<COUNT, true, false>)
+                                : (plates ? k_irradiance<COUNT, false, !COUNT> : k_irradiance<COUNT, false, false>);
+    const void* kern = (const void*)kernel;
     int rc = allow_smem(kern, smem);
     if (rc != UVC_OK) return rc;
     const int njb = (S.np + 31) / 32;
     const int64_t ntask = ((nc + kCandPerTask - 1) / kCandPerTask) * njb;
     int grid = grid_for(kern, smem);
     if ((int64_t)grid * kWarpsPerBlock > ntask) grid = (int)((ntask + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    if (wedge)
-        k_irradiance<COUNT, true><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, A, lda, vis, ctr);
-    else
-        k_irradiance<COUNT, false><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, A, lda, vis, ctr);
+    kernel<<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, A, lda, vis, ctr);
     return status_from_cuda(cudaGetLastError());
 }
 

@@ -251,11 +251,12 @@ __global__ void k_plate_check(const float4* __restrict__ tri, int nt, int* __res
 
 // The plates, in any order (no result depends on it); their number may pass
 // kMaxPlates, and the scene then goes without.  plate_id: per root, or -1.
+// box: the scene's bounds; inner: triangles of the plates inside them.
 __global__ void k_plate_select(const float4* __restrict__ tri, int nt, const int* __restrict__ parent,
                                const uint2* __restrict__ lo, const uint2* __restrict__ hi,
                                const int2* __restrict__ cnt_bad, const unsigned* __restrict__ len,
                                const float* __restrict__ area2, float4* __restrict__ plates, int* __restrict__ plate_id,
-                               int* __restrict__ nplate) {
+                               const unsigned* __restrict__ box, int* __restrict__ nplate, int* __restrict__ inner) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nt) return;
     int id = -1;
@@ -264,6 +265,7 @@ __global__ void k_plate_select(const float4* __restrict__ tri, int nt, const int
         id = atomicAdd(nplate, 1);
         if (id < kMaxPlates) {
             const Flat f = flat_of(tri, k);
+            if (f.p > unordered(box[f.axis]) && f.p < unordered(box[3 + f.axis])) atomicAdd(inner, cnt_bad[k].x);
             const int i = f.axis == 2 ? 0 : f.axis + 1, j = i == 2 ? 0 : i + 1;
             float a[3], b[3];
             a[f.axis] = b[f.axis] = f.p;
@@ -341,10 +343,12 @@ size_t plates_work_bytes(int64_t nt) {
 
 // Enqueues the search for the scene's plates (see above): sc->plates and the
 // patch flags, counts[0] = plates found (may pass kMaxPlates), counts[1] =
-// loose triangles (both zeroed by the caller), and the loose marks of leaves
-// and binary nodes (node_loose zeroed by the caller).
+// loose triangles, counts[2] = triangles of plates inside the scene's bounds
+// (all zeroed by the caller), and the loose marks of leaves and binary nodes
+// (node_loose zeroed by the caller).  box: the triangles' bounds, lo and hi, as
+// ordered integers.
 void find_plates(uvc_scene* sc, const int* parent_leaf, const int* parent_int, int* leaf_loose, int* node_loose,
-                 int* counts, void* work, cudaStream_t stream) {
+                 const unsigned* box, int* counts, void* work, cudaStream_t stream) {
     const int nt = (int)sc->nt, np = (int)sc->np;
     const uint32_t slots = table_slots(nt);
     char* p = static_cast<char*>(work);
@@ -365,7 +369,8 @@ void find_plates(uvc_scene* sc, const int* parent_leaf, const int* parent_int, i
     k_plate_edges<<<grid(4 * (int64_t)nt), 256, 0, stream>>>(sc->tri, nt, table, slots - 1, parent, state);
     k_plate_stats<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, state, lo, hi, cnt_bad, len, area2);
     k_plate_check<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, state, lo, hi, cnt_bad);
-    k_plate_select<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, lo, hi, cnt_bad, len, area2, sc->plates, plate_id, counts);
+    k_plate_select<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, lo, hi, cnt_bad, len, area2, sc->plates, plate_id,
+                                                 box, counts, counts + 2);
     k_plate_mark<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, plate_id, parent_leaf, parent_int, sc->tri_place,
                                                leaf_loose, node_loose, counts + 1);
     if (np > 0)

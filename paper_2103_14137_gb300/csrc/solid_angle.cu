@@ -185,8 +185,8 @@ __device__ __forceinline__ uint32_t packet_to(const SceneView& S, float ox, floa
 // search for all of a candidate's sources that still need it (see the wedge
 // traversal in traverse.cuh); the per-source results, and so the entries, are
 // those of the source-by-source searches.
-template <bool WEDGE>
-__global__ void __launch_bounds__(kThreads, kCallMinBlocks)
+template <bool WEDGE, bool PLATES>
+__global__ void __launch_bounds__(kThreads, PLATES ? kCallMinBlocks : UVC_IRR_MIN_BLOCKS)
     k_area_mean(const __grid_constant__ SceneView S, const float* __restrict__ cand, int nc, const __grid_constant__ LampDev L, const float* __restrict__ ptri,
                 float* __restrict__ A, int64_t lda, uint8_t* __restrict__ nclosed, const int2* __restrict__ tri_place, int cpt) {
     extern __shared__ __align__(16) int smem[];
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, kCallMinBlocks)
         const int j = jb * 32 + lane;
         const PatchLane P = load_patch(S, j);
         const float* g = ptri + 18 * (size_t)(P.valid ? j : 0);
-        const PlateLane pl = WEDGE && S.nplate != 0 ? plate_lane(S, jb, lane, P) : no_plate_lane();
+        const PlateLane pl = PLATES && S.nplate != 0 ? plate_lane(S, jb, lane, P) : no_plate_lane();
         const int tmask = used_triangles(g, P.valid);
         const float inv_area = P.valid && P.s.w > 0.f ? __frcp_rn(P.s.w) : 0.f;
         int cache = -1;
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, kCallMinBlocks)
         float gap[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         PlateLane plc = pl;
         plc.plate = -1;
-        if (WEDGE && S.nplate != 0 && L.plates && pl.own_axis >= 0) {
+        if (PLATES && S.nplate != 0 && L.plates && pl.own_axis >= 0) {
             float2 T[2][3];
             bool in[2] = {false, false};
             const int ax = pl.own_axis;
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, kCallMinBlocks)
                         if (!(plq.gap > 0.f)) plq.own_axis = -1;
                     }
                     uint32_t fq;
-                    const uint32_t oc = wedge_search<false, true>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex, plq, lane, stack, ws, cache, fq, nullptr);
+                    const uint32_t oc = wedge_search<false, PLATES, PLATES>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex, plq, lane, stack, ws, cache, fq, nullptr);
                     failed_all |= fq;
                     if (q < 0) {
                         vis_c = ((fq >> lane) & 1u) ? 0u : (facing & ~oc);
@@ -370,7 +370,11 @@ int irradiance_area_mean(const uvc_scene* sc, const float* cand, int64_t nc, con
     SceneView S = view_of(sc);
     const bool wedge = lamp.wedge != 0;
     const size_t smem = stack_smem_bytes(S.stack_cap) + (wedge ? wedge_smem_bytes(lamp.K) : 0);
-    const void* kern = wedge ? (const void*)k_area_mean<true> : (const void*)k_area_mean<false>;
+    using Kernel = void (*)(const SceneView, const float*, int, const LampDev, const float*, float*, int64_t, uint8_t*,
+                            const int2*, int);
+    const Kernel kernel = wedge ? (S.nplate != 0 && lamp.plates ? k_area_mean<true, true> : k_area_mean<true, false>)
+                                : k_area_mean<false, false>;
+    const void* kern = (const void*)kernel;
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return status_from_cuda(e);
@@ -384,10 +388,7 @@ int irradiance_area_mean(const uvc_scene* sc, const float* cand, int64_t nc, con
     const int cpt = (int)std::max<int64_t>(kAreaCandMin, std::min<int64_t>(kAreaCandMax, per_warp / 8));
     const int64_t ntask = ((nc + cpt - 1) / cpt) * njb;
     if ((int64_t)grid * kWarpsPerBlock > ntask) grid = (int)((ntask + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    if (wedge)
-        k_area_mean<true><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, ptri, A, lda, nclosed, sc->tri_place, cpt);
-    else
-        k_area_mean<false><<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, ptri, A, lda, nclosed, sc->tri_place, cpt);
+    kernel<<<grid, kThreads, smem, stream>>>(S, cand, (int)nc, lamp, ptri, A, lda, nclosed, sc->tri_place, cpt);
     return status_from_cuda(cudaGetLastError());
 }
 

@@ -637,7 +637,7 @@ __device__ __forceinline__ PlateLane plate_lane(const SceneView& S, int jb, int 
 // `cache` is the lane's last occluding triangle (sorted index, -1 = none): it
 // is tested first, and a hit settles the segment without a traversal (the
 // same predicate the traversal would apply to that triangle).
-template <bool COUNT = false>
+template <bool COUNT, bool PLATES>
 __device__ __forceinline__ float irradiance_entry(const SceneView& S, const float* __restrict__ cand, int nc,
                                                   const LampDev& L, int i, int jb, int lane, int* stack,
                                                   uint32_t* __restrict__ vis, int nwords, const PatchLane& P,
@@ -645,7 +645,7 @@ __device__ __forceinline__ float irradiance_entry(const SceneView& S, const floa
     const float4 s4 = P.s, n4 = P.n;
     const float cx = __ldg(&cand[3 * (size_t)i]), cy = __ldg(&cand[3 * (size_t)i + 1]),
                 cz = __ldg(&cand[3 * (size_t)i + 2]);
-    const bool plates = !COUNT && S.nplate != 0 && L.plates;
+    const bool plates = PLATES && S.nplate != 0 && L.plates;
     const PlateLane pl = plates ? plate_lane(S, jb, lane, P) : no_plate_lane();
     float E = 0.f;
     bool bad = false;
@@ -1335,8 +1335,10 @@ __device__ __noinline__ WedgeRest wedge_rest_call(const SceneView& S, const Lamp
 // The search from the lamp line of candidate c to the lane's point (height sz,
 // horizontal direction (gx, gy) from c) for the sources in `want`: the plates
 // first, then the hierarchy for what they leave.  Returns the sources found
-// occluded; `failed` as in wedge_rest.  CALL: wedge_rest is called, not inlined.
-template <bool COUNT, bool CALL>
+// occluded; `failed` as in wedge_rest.  PLATES: compiled with the plate tests
+// (scenes without plates take kernels without them: their registers cost a
+// tilted room 4 to 20 %).  CALL: wedge_rest is called, not inlined.
+template <bool COUNT, bool PLATES, bool CALL>
 __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampDev& L, float cx, float cy, float cz,
                                                  float sz, float gx, float gy, uint32_t want, float lend, float dmax,
                                                  int2 ex, const PlateLane& pl, int lane, int* stack, const WedgeSmem& ws,
@@ -1344,7 +1346,7 @@ __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampD
     failed = 0;
     if (S.nt == 0 || !__any_sync(kFull, want != 0u)) return 0u;
     const uint32_t before = want;
-    const bool plates = !COUNT && S.nplate != 0 && L.plates;
+    const bool plates = PLATES && S.nplate != 0 && L.plates;
     const Slabs sl = slabs_of(cx, cy, gx, gy, S.cut_eps);
     uint32_t open = want;
     if (plates) {
@@ -1379,7 +1381,7 @@ __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampD
 // Irradiance of candidate i at this lane's patch for a vertical line lamp
 // (L.wedge): the same entry as irradiance_entry, with one search per candidate
 // instead of one per source.
-template <bool COUNT = false, bool MODES = false, bool CALL = false>
+template <bool COUNT, bool PLATES, bool MODES, bool CALL>
 __device__ __forceinline__ float irradiance_wedge(const SceneView& S, const float* __restrict__ cand, int nc,
                                                   const LampDev& L, int i, int jb, int lane, int* stack,
                                                   const WedgeSmem& ws, uint32_t* __restrict__ vis, int nwords,
@@ -1391,8 +1393,8 @@ __device__ __forceinline__ float irradiance_wedge(const SceneView& S, const floa
     float E;
     const uint32_t facing = wedge_setup_patch<MODES>(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, E);
     uint32_t failed;
-    const PlateLane pl = !COUNT && S.nplate != 0 ? plate_lane(S, jb, lane, P) : no_plate_lane();
-    const uint32_t occl = wedge_search<COUNT, CALL>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, pl, lane,
+    const PlateLane pl = PLATES && S.nplate != 0 ? plate_lane(S, jb, lane, P) : no_plate_lane();
+    const uint32_t occl = wedge_search<COUNT, PLATES, CALL>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, pl, lane,
                                               stack, ws, cache, failed, ctr);
     const bool bad = (failed >> lane) & 1u;
     const uint32_t visible = bad ? 0u : (facing & ~occl);

@@ -122,7 +122,7 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
 // plates (plates.cu)
 size_t plates_work_bytes(int64_t nt);
 void find_plates(uvc_scene* sc, const int* parent_leaf, const int* parent_int, int* leaf_loose, int* node_loose,
-                 int* counts, void* work, cudaStream_t stream);
+                 const unsigned* box, int* counts, void* work, cudaStream_t stream);
 
 // irradiance (irradiance.cu)
 int irradiance_matrix(const uvc_scene* sc, const float* cand, int64_t nc, const LampDev& lamp, float* A,

@@ -66,6 +66,10 @@ def _scenes():
         "t_junction": (np.concatenate([room, _face([1, 1, 1], [1, 0, 0], [0, 1, 0], 2, 2),
                                        _face([2, 1, 1], [1, 0, 0], [0, 0.5, 0], 2, 1),
                                        _face([2, 1.5, 1], [1, 0, 0], [0, 0.5, 0], 2, 2)]), True),
+        # the scene keeps its plates while the loose triangles are at most 8 times the 48 of the inner ones
+        "loose_at_the_line": (np.concatenate([room, _box([1, 1, 0.25], [2, 2, 0.75], 2), _face([2.2, 1, 0.5], [1, 0, 0.2], [0, 1, 0], 12, 16)]), True),
+        "loose_over_the_line": (np.concatenate([room, _box([1, 1, 0.25], [2, 2, 0.75], 2), _face([2.2, 1, 0.5], [1, 0, 0.2], [0, 1, 0], 193, 1)]), True),
+        "walls_and_turned_box": (np.concatenate([room, _box([1.4, 0.6, 0.1], [3.2, 1.3, 1.5], 3, 1, 0.4)]), True),
         "thin_triangles": (np.concatenate([room, _face([1, 1, 1], [1.5, 0, 0], [0, 0.5, 0], 1, 40)]), True),
         "over_32_plates": (np.concatenate([room] + [_box([0.3 + 0.5 * i, 0.4 + 0.6 * j, 0.1], [0.6 + 0.5 * i, 0.7 + 0.6 * j, 0.5 + 0.2 * j], 2)
                                                     for i in range(7) for j in range(4)]), False),
