@@ -53,6 +53,7 @@ int lamp_to_device(const uvc_lamp* lamp, LampDev* out, float coord_bound, int64_
         out->oz[m] = lamp->offsets[m][2];
         out->pw[m] = per_4pi ? (float)((double)w * (double)lamp->power / (4.0 * M_PI)) : w * lamp->power;
     }
+    if (lamp->K < UVC_MAX_SOURCES) out->oz[lamp->K] = out->oz[lamp->K - 1];   // pw = 0 there
     out->zmin = out->zmax = out->oz[0];
     for (int m = 1; m < lamp->K; ++m) {
         out->zmin = std::min(out->zmin, out->oz[m]);

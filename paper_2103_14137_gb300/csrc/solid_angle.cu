@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, PLATES ? kCallMinBlocks : UVC_IRR_MI
                         if (!(plq.gap > 0.f)) plq.own_axis = -1;
                     }
                     uint32_t fq;
-                    const uint32_t oc = wedge_search<false, PLATES, PLATES>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex, plq, lane, stack, ws, cache, fq, nullptr);
+                    const uint32_t oc = wedge_search<false, PLATES, PLATES, PLATES>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex, plq, lane, stack, ws, cache, fq, nullptr);
                     failed_all |= fq;
                     if (q < 0) {
                         vis_c = ((fq >> lane) & 1u) ? 0u : (facing & ~oc);

@@ -501,11 +501,11 @@ __device__ __forceinline__ PlateLane no_plate_lane() { return PlateLane{false, -
 // parameter a search would look at, dmax the longest segment.  Takes the
 // blocked sources out of `want` and returns the open ones among the rest (the
 // others are clear of every plate).  Every lane of the warp calls it.
-template <class Z>
+template <bool ENDS, class Z>
 __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, int K, float cx, float cy, float sz,
                                                   float gx, float gy, float zlo, float zhi, float lend, float dmax,
                                                   const Slabs& sl, const PlateLane& pl, int lane, uint32_t& want) {
-    const float kBig = 3.0e38f;
+    const float kBig = 3.0e38f, kWide = 4.76837158203125e-07f;   // 2^-21: the rounding of a rectangle's middle and half width
     const bool a0 = want != 0u;
     const float delta = S.cut_eps, diag = S.cut_eps * 1e5f;
     // far outside the scene (or infinite, or NaN) the widening no longer covers the rounding of the shaft
@@ -572,34 +572,64 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
                         const float gb = isx ? gy : gx, hs = ho + ga;
                         const float lb = isx ? lo.y - cy : lo.x - cx, ub = isx ? hi.y - cy : hi.x - cx;
                         if (fminf(fabsf(ho), fabsf(hs)) >= far_off) {
-                            const float lam = -ho * ig, m = near_in * dmax * fabsf(ig);
-                            const float t = fabsf(fmaf(lam, gb, -0.5f * (lb + ub))) - 0.5f * (ub - lb);
+                            const float lam = -ho * ig, mid = 0.5f * (lb + ub), half = 0.5f * (ub - lb);
+                            const float m0 = near_in * dmax * fabsf(ig), m = fmaf(fabsf(mid) + half, kWide, m0);
+                            const float t = fabsf(fmaf(lam, gb, -mid)) - half;
                             if (ho * hs > 0.f || t > m) {
                                 clear = want;
                             } else {
                                 const bool inside = t < -m;
-                                const float hz = 0.5f * (hi.z - lo.z), zc = fmaf(lam, sz, -0.5f * (lo.z + hi.z));
-                                for (int q = 0; q < K; ++q) {
-                                    const float tz = fabsf(fmaf(1.f - lam, zsrc(q), zc)) - hz;
-                                    if (tz > m) clear |= 1u << q;
-                                    else if (inside && tz < -m) blocked |= 1u << q;
+                                const float lz = lo.z - sz, uz = hi.z - sz, mu = 1.f - lam;
+                                const float mz = 0.5f * (lz + uz), hz = 0.5f * (uz - lz);
+                                const float w = fmaf(fabsf(mz) + hz, kWide, m0);
+                                const float e0 = fmaf(mu, zlo - sz, -mz), e1 = fmaf(mu, zhi - sz, -mz);
+                                if (ENDS && fmaxf(-e1, e0) - hz > w) clear = want;
+                                else if (ENDS && inside && fmaxf(-e0, e1) - hz < -w) blocked = want;
+                                else for (int q = 0; q < K; ++q) {
+                                    const float tz = fabsf(fmaf(mu, zsrc(q) - sz, -mz)) - hz;
+                                    if (tz > w) clear |= 1u << q;
+                                    else if (inside && tz < -w) blocked |= 1u << q;
                                 }
                             }
                         }
                     } else {
                         const float hs = sz - lo.z;
-                        const float xc = cx - 0.5f * (lo.x + hi.x), yc = cy - 0.5f * (lo.y + hi.y);
-                        const float hx = 0.5f * (hi.x - lo.x), hy = 0.5f * (hi.y - lo.y);
-                        if (fabsf(hs) >= far_off)
-                            for (int q = 0; q < K; ++q) {
-                                const float hm = zsrc(q) - lo.z, dz = hm - hs;
-                                if (fabsf(hm) >= far_off) {
-                                    const float ig = rcp_approx(dz), lam = hm * ig, m = near_in * dmax * fabsf(ig);
-                                    const float t = fmaxf(fabsf(fmaf(lam, gx, xc)) - hx, fabsf(fmaf(lam, gy, yc)) - hy);
-                                    if (hm * hs > 0.f || t > m) clear |= 1u << q;
-                                    else if (t < -m) blocked |= 1u << q;
+                        const float lx = lo.x - cx, ux_ = hi.x - cx, ly = lo.y - cy, uy_ = hi.y - cy;
+                        const float xc = 0.5f * (lx + ux_), hx = 0.5f * (ux_ - lx), yc = 0.5f * (ly + uy_), hy = 0.5f * (uy_ - ly);
+                        const float wide = fmaxf(fabsf(xc) + hx, fabsf(yc) + hy) * kWide;
+                        if (fabsf(hs) >= far_off) {
+                            bool done = false;
+                            if (ENDS) {   // both ends of the lamp on one side; the crossing points lie on a line between theirs
+                                const float h0 = zlo - lo.z, h1 = zhi - lo.z;
+                                const bool off = fminf(fabsf(h0), fabsf(h1)) >= far_off;
+                                if (fminf(h0 * hs, h1 * hs) > 0.f) {
+                                    done = off;
+                                    if (off) clear = want;
+                                } else if (off && fmaxf(h0 * hs, h1 * hs) < 0.f) {
+                                    const float i0 = rcp_approx(h0 - hs), i1 = rcp_approx(h1 - hs);
+                                    const float m = fmaf(near_in * dmax, fmaxf(fabsf(i0), fabsf(i1)), wide);
+                                    const float xa = fmaf(h0 * i0, gx, -xc), xb = fmaf(h1 * i1, gx, -xc);
+                                    const float ya = fmaf(h0 * i0, gy, -yc), yb = fmaf(h1 * i1, gy, -yc);
+                                    const float away = fmaxf(fmaxf(fminf(xa, xb), -fmaxf(xa, xb)) - hx,
+                                                             fmaxf(fminf(ya, yb), -fmaxf(ya, yb)) - hy);
+                                    const float in_ = fmaxf(fmaxf(fabsf(xa), fabsf(xb)) - hx, fmaxf(fabsf(ya), fabsf(yb)) - hy);
+                                    done = away > m || in_ < -m;
+                                    if (away > m) clear = want;
+                                    else if (in_ < -m) blocked = want;
                                 }
                             }
+                            if (!done)
+                                for (int q = 0; q < K; ++q) {
+                                    const float hm = zsrc(q) - lo.z, dz = hm - hs;
+                                    if (fabsf(hm) >= far_off) {
+                                        const float ig = rcp_approx(dz), lam = hm * ig;
+                                        const float m = fmaf(near_in * dmax, fabsf(ig), wide);
+                                        const float t = fmaxf(fabsf(fmaf(lam, gx, -xc)) - hx, fabsf(fmaf(lam, gy, -yc)) - hy);
+                                        if (hm * hs > 0.f || t > m) clear |= 1u << q;
+                                        else if (t < -m) blocked |= 1u << q;
+                                    }
+                                }
+                        }
                     }
                     if (pl.flagged) blocked = 0u;
                     open |= want & ~(blocked | clear);
@@ -663,7 +693,7 @@ __device__ __forceinline__ float irradiance_entry(const SceneView& S, const floa
         uint32_t want = facing && !(tend <= 0.f) ? 1u : 0u, open = want, found = 0u, failed = 0u;
         const uint32_t before = want;
         if (plates && __any_sync(kFull, want))
-            open = plates_decide(S, [&](int) { return oz; }, 1, ox, oy, s4.z, -hx, -hy, oz, oz,
+            open = plates_decide<false>(S, [&](int) { return oz; }, 1, ox, oy, s4.z, -hx, -hy, oz, oz,
                                  tend, d, slabs_of(ox, oy, -hx, -hy, S.cut_eps), pl, lane, want);
         for (int whole = plates && (S.nplate & kLooseBit) ? 0 : 1; whole < 2; ++whole) {
             const uint32_t search = __ballot_sync(kFull, want && (whole ? open : !open));
@@ -1119,22 +1149,18 @@ __device__ __forceinline__ uint32_t wedge_setup_patch(const SceneView& S, const 
     uint32_t facing = 0;
     float far2 = 0.f;
     sum = 0.f;
-    // One pass over the pairs of sources.  NORMAL: 0 = any normal; 1 = horizontal
-    // normals (n.z = 0), where <n, v> is the same for all sources; 2 = vertical
-    // ones, where it is n.z times the rounded height difference (the rounded sum
-    // of a rounded difference and its error is that difference).  Each gives what
-    // the general form does.
-    auto pass = [&](auto normal) {
-        constexpr int NORMAL = decltype(normal)::value;
-        const float nv0 = __fadd_rn(acc0, err0);
+    // One pass over the pairs of sources.  VERTICAL: for vertical normals, where
+    // <n, v> is n.z times the rounded height difference (the rounded sum of a
+    // rounded difference and its error is that difference): what the general
+    // form gives.
+    auto pass = [&](auto vertical) {
+        constexpr bool VERTICAL = decltype(vertical)::value;
         for (int m = 0; m < L.K; m += 2) {
             const int k = min(m + 1, L.K - 1);   // an odd lamp's last source twice; its second half is dropped
             const float2 oz = __fadd2_rn(c2, make_float2(L.oz[m], L.oz[k]));
             const float2 hz = sub2(oz, sz, m1);
             float2 nv;
-            if constexpr (NORMAL == 1) {
-                nv = dup2(nv0);
-            } else if constexpr (NORMAL == 2) {
+            if constexpr (VERTICAL) {
                 nv = __fmul2_rn(nz, hz);
             } else {
                 const float2 qz = sub2(hz, oz, m1);
@@ -1164,10 +1190,47 @@ __device__ __forceinline__ uint32_t wedge_setup_patch(const SceneView& S, const 
             facing |= ((uint32_t)f0 << m) | ((uint32_t)f1 << k);
         }
     };
-    const bool hor = n4.z == 0.f, ver = n4.x == 0.f && n4.y == 0.f && fabsf(n4.z) == 1.f;
-    if (MODES && __all_sync(kFull, hor || !P.valid)) pass(std::integral_constant<int, 1>());
-    else if (MODES && __all_sync(kFull, ver || !P.valid)) pass(std::integral_constant<int, 2>());
-    else pass(std::integral_constant<int, 0>());
+    if constexpr (MODES) {
+        // Horizontal normals (n.z = 0), where <n, v> is the same for all sources,
+        // and vertical ones whose lamp is all above or all below: every source
+        // faces or none does, and distances are extreme at the lamp's ends (each
+        // step of d2 is monotonic under rounding).
+        const bool hor = n4.z == 0.f, ver = n4.x == 0.f && n4.y == 0.f && fabsf(n4.z) == 1.f;
+        const float hl = __fsub_rn(__fadd_rn(cz, L.zmin), s4.z), hh = __fsub_rn(__fadd_rn(cz, L.zmax), s4.z);
+        const float he = fmaxf(-hl, hh), hm = fmaxf(fmaxf(hl, -hh), 0.f);   // largest and least distance in z
+        const float dmin = __fmaf_rn(hx, hx, __fmaf_rn(hy, hy, __fmul_rn(hm, hm)));
+        const float n0 = hor ? __fadd_rn(acc0, err0) : 0.f, n1 = hor ? 0.f : n4.z;
+        const bool up = __fmaf_rn(n1, hl, n0) > 0.f, down = __fmaf_rn(n1, hh, n0) > 0.f;
+        far2 = __fmaf_rn(hx, hx, __fmaf_rn(hy, hy, __fmul_rn(he, he)));
+        const bool ordinary = dmin >= kTermMin && far2 <= kTermMax;
+        const bool simple = __all_sync(kFull, !P.valid || ((hor || ver) && up == down && ordinary));
+        if (simple) {
+            const bool face = P.valid && up;
+            if (__any_sync(kFull, face)) {
+                const float2 b = dup2(n0), nzs = dup2(n1);
+                for (int m = 0; m < L.K; m += 2) {
+                    const float2 hz = sub2(__fadd2_rn(c2, *reinterpret_cast<const float2*>(&L.oz[m])), sz, m1);
+                    const float2 nv = __ffma2_rn(nzs, hz, b);
+                    const float2 d2 = __ffma2_rn(hx2, hx2, __ffma2_rn(hy2, hy2, __fmul2_rn(hz, hz)));
+                    const float2 r = make_float2(rsqrt_approx(d2.x), rsqrt_approx(d2.y));
+                    const float2 r2 = __fmul2_rn(r, r), r3 = __fmul2_rn(r2, r), f = __ffma2_rn(d2, r2, m1);
+                    const float2 w = __ffma2_rn(__fmul2_rn(f, make_float2(-1.5f, -1.5f)), r3, r3);
+                    const float2 t = __fmul2_rn(*reinterpret_cast<const float2*>(&L.pw[m]), __fmul2_rn(nv, w));
+                    ws.term[m * 32 + lane] = t.x;
+                    if (m + 1 < L.K) ws.term[(m + 1) * 32 + lane] = t.y;
+                    sum = __fadd_rn(__fadd_rn(sum, t.x), t.y);   // an odd lamp's extra half adds 0
+                }
+            }
+            sum = face ? sum : 0.f;
+            facing = face ? (1u << L.K) - 1u : 0u;
+        } else {
+            far2 = 0.f;
+            if (__all_sync(kFull, ver || !P.valid)) pass(std::true_type());
+            else pass(std::false_type());
+        }
+    } else {
+        pass(std::false_type());
+    }
     if (!P.valid) facing = 0u;
     gx = -hx;
     gy = -hy;
@@ -1338,7 +1401,7 @@ __device__ __noinline__ WedgeRest wedge_rest_call(const SceneView& S, const Lamp
 // occluded; `failed` as in wedge_rest.  PLATES: compiled with the plate tests
 // (scenes without plates take kernels without them: their registers cost a
 // tilted room 4 to 20 %).  CALL: wedge_rest is called, not inlined.
-template <bool COUNT, bool PLATES, bool CALL>
+template <bool COUNT, bool PLATES, bool ENDS, bool CALL>
 __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampDev& L, float cx, float cy, float cz,
                                                  float sz, float gx, float gy, uint32_t want, float lend, float dmax,
                                                  int2 ex, const PlateLane& pl, int lane, int* stack, const WedgeSmem& ws,
@@ -1360,7 +1423,7 @@ __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampD
                 zhi = fmaxf(zhi, oz);
             }
         }
-        open = plates_decide(S, [&](int q) { return __fadd_rn(cz, L.oz[q]); }, L.K, cx, cy, sz, gx, gy, zlo, zhi, lend,
+        open = plates_decide<ENDS>(S, [&](int q) { return __fadd_rn(cz, L.oz[q]); }, L.K, cx, cy, sz, gx, gy, zlo, zhi, lend,
                              dmax, sl, pl, lane, want);
     }
     if (CALL) {
@@ -1394,7 +1457,7 @@ __device__ __forceinline__ float irradiance_wedge(const SceneView& S, const floa
     const uint32_t facing = wedge_setup_patch<MODES>(S, L, cx, cy, cz, P, lane, ws, want, lend, dmax, gx, gy, E);
     uint32_t failed;
     const PlateLane pl = PLATES && S.nplate != 0 ? plate_lane(S, jb, lane, P) : no_plate_lane();
-    const uint32_t occl = wedge_search<COUNT, PLATES, CALL>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, pl, lane,
+    const uint32_t occl = wedge_search<COUNT, PLATES, MODES, CALL>(S, L, cx, cy, cz, P.s.z, gx, gy, want, lend, dmax, P.ex, pl, lane,
                                               stack, ws, cache, failed, ctr);
     const bool bad = (failed >> lane) & 1u;
     const uint32_t visible = bad ? 0u : (facing & ~occl);

@@ -66,7 +66,8 @@ struct LampDev {
     int wuniform;
     float wz0, wrdz;
     float zmin, zmax;
-    float ox[UVC_MAX_SOURCES], oy[UVC_MAX_SOURCES], oz[UVC_MAX_SOURCES];
+    alignas(8) float ox[UVC_MAX_SOURCES];   // aligned: sources are read in pairs
+    float oy[UVC_MAX_SOURCES], oz[UVC_MAX_SOURCES];   // oz: an odd lamp's last entry twice
     float pw[UVC_MAX_SOURCES];
 };
 

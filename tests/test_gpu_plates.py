@@ -122,6 +122,19 @@ def test_plates_give_the_search_results(name):
     sc.free()
 
 
+@pytest.mark.parametrize("shift", [(64.0, -32.0, 16.0), (-300.0, 500.0, 100.0)])
+@pytest.mark.parametrize("name", ["plates_only", "over_32_plates"])
+def test_plates_far_from_the_origin(name, shift):
+    """The decisions rest on differences of coordinates, as the search's triangle tests do."""
+    T, _ = _scenes()[name]
+    (verts, tris, cen, nrm, excl), _, cand = _patches(T, name)
+    verts, cen, cand = (np.float32(x + np.float32(shift)) for x in (verts, cen, cand))
+    sc = build_arrays(verts, tris, cen, nrm, np.ones(300, np.float32), excl)
+    for L in _lamps().values():
+        _same_as_per_source((verts, tris, cen, nrm, excl), sc, cand, L)
+    sc.free()
+
+
 @pytest.mark.parametrize("name", ["plates_only", "window_in_a_wall", "doubled_triangle", "over_32_plates"])
 @pytest.mark.parametrize("lamp", ["line2", "line16"])
 def test_area_mean_at_plates_gives_the_search_results(name, lamp):
