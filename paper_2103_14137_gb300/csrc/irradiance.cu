@@ -84,14 +84,20 @@ __global__ void __launch_bounds__(kThreads, UVC_IRR_MIN_BLOCKS) k_irradiance(Sce
 // E values of up to kStreamedBlock candidates are staged in shared memory,
 // multiplied by the dwell times and added to the chunk's partial sums
 // partial[s][v][j].  20 candidates per stage keeps a K = 8 lamp's block within
-// a third of an SM's shared memory (three resident blocks).  A task is a whole
+// a third of an SM's shared memory.  The weighting was bound by shared memory and
+// L1 (two loads for each multiply): with the E values in registers and the
+// dwell times read four at a time a floor of rooms (266 k patches, 250
+// candidates, 64 plans) takes 2.93 ms instead of 3.82, and 2.67 with the set-up
+// passes by surface, the hierarchy search as a call and two blocks per SM (a
+// point lamp, and scenes without plates: three blocks).  A task is a whole
 // chunk of candidates for 32 patches, and its cost varies with the geometry
 // around the patches, so the warps take tasks from a counter (next_task,
 // zeroed before the launch) as they finish instead of a fixed share each;
 // every task's sums are the same whichever warp takes it.
 constexpr int kStreamedBlock = 20;
+static_assert(kStreamedBlock % 4 == 0, "rows of dwell times are read four at a time");
 template <bool WEDGE, bool PLATES>
-__global__ void __launch_bounds__(kThreads, UVC_STREAMED_MIN_BLOCKS) k_streamed(SceneView S, const float* __restrict__ cand, int nc,
+__global__ void __launch_bounds__(kThreads, WEDGE && PLATES ? kCallMinBlocks : UVC_STREAMED_MIN_BLOCKS) k_streamed(SceneView S, const float* __restrict__ cand, int nc,
                                                        LampDev L, const float* __restrict__ t, int nvec,
                                                        float* __restrict__ partial, int nsplit, int chunk,
                                                        unsigned long long* next_task) {
@@ -119,16 +125,39 @@ __global__ void __launch_bounds__(kThreads, UVC_STREAMED_MIN_BLOCKS) k_streamed(
             const int nb = min(kStreamedBlock, i1 - ib);
             for (int q = 0; q < nb; ++q)
                 Et[q * 32 + lane] =
-                    WEDGE ? irradiance_wedge<false, PLATES, false, false>(S, cand, nc, L, ib + q, jb, lane, stack, ws, nullptr, 0, P, cache)
+                    WEDGE ? irradiance_wedge<false, PLATES, PLATES, PLATES>(S, cand, nc, L, ib + q, jb, lane, stack, ws, nullptr, 0, P, cache)
                           : irradiance_entry<false, PLATES>(S, cand, nc, L, ib + q, jb, lane, stack, nullptr, 0, P, cache);
-            __syncwarp();
-            if (j < S.np) {
-                for (int v = 0; v < nvec; ++v) {
-                    const float* tv = t + (size_t)v * nc + ib;
-                    float sum = 0.f;
-                    for (int q = 0; q < nb; ++q) sum = __fmaf_rn(__ldg(tv + q), Et[q * 32 + lane], sum);
-                    float* pp = partial + ((size_t)s * nvec + v) * S.np + j;
-                    *pp = (ib == i0) ? sum : __fadd_rn(*pp, sum);
+            // The lane's E values move to registers and their place takes the dwell
+            // times of up to 32 vectors at a time, read back four at a time by all
+            // lanes; rows past nb are 0 and leave the sums as they are.
+            float e[kStreamedBlock];
+#pragma unroll
+            for (int q = 0; q < kStreamedBlock; ++q) e[q] = q < nb ? Et[q * 32 + lane] : 0.f;
+            float* pp = partial + (size_t)s * nvec * S.np + j;
+            for (int v0 = 0; v0 < nvec; v0 += 32) {
+                const int nv = min(32, nvec - v0);
+                __syncwarp();
+                for (int k = lane; k < nv * kStreamedBlock; k += 32) {
+                    const int v = k / kStreamedBlock, q = k - v * kStreamedBlock;
+                    Et[k] = q < nb ? __ldg(t + (size_t)(v0 + v) * nc + ib + q) : 0.f;
+                }
+                __syncwarp();
+                if (j < S.np) {
+#pragma unroll 4
+                    for (int v = 0; v < nv; ++v, pp += S.np) {
+                        const float4* row = reinterpret_cast<const float4*>(Et + v * kStreamedBlock);
+                        const float before = ib == i0 ? 0.f : *pp;
+                        float sum = 0.f;
+#pragma unroll
+                        for (int q = 0; q < kStreamedBlock / 4; ++q) {
+                            const float4 w = row[q];
+                            sum = __fmaf_rn(w.x, e[4 * q], sum);
+                            sum = __fmaf_rn(w.y, e[4 * q + 1], sum);
+                            sum = __fmaf_rn(w.z, e[4 * q + 2], sum);
+                            sum = __fmaf_rn(w.w, e[4 * q + 3], sum);
+                        }
+                        *pp = ib == i0 ? sum : __fadd_rn(before, sum);
+                    }
                 }
             }
             __syncwarp();

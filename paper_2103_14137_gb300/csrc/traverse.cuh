@@ -1118,8 +1118,7 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b, float2 m1) { return _
 // clearance cut), with the largest cut parameter `lend`, the longest such
 // segment `dmax` and the common horizontal direction (gx, gy).
 // MODES: separate passes for horizontal and vertical normals (the walls, floors
-// and ceilings of rooms: ward matrix 8.6 -> 8.1 ms).  They cost registers that
-// the streamed kernel does not have (3.9 -> 5.4 ms there).
+// and ceilings of rooms: ward matrix 8.6 -> 8.1 ms, 7.5 with the whole-lamp form).
 template <bool MODES>
 __device__ __forceinline__ uint32_t wedge_setup_patch(const SceneView& S, const LampDev& L, float cx, float cy,
                                                       float cz, const PatchLane& P, int lane, const WedgeSmem& ws,
@@ -1375,8 +1374,9 @@ __device__ __forceinline__ uint32_t wedge_rest(const SceneView& S, const LampDev
 // batch's job records, the area mean's patches and gaps): on a room of plates a
 // packet in a hundred gets there.  Measured with 128 registers (two blocks per SM):
 // batched rooms 3.09 -> 2.71 ms, area mean 4.08 -> 3.56 ms; inlined at two blocks
-// 3.07 and 3.83.  The plain and streamed kernels are faster with it inlined at
-// three blocks (ward matrix 8.1 against 8.6 ms, streamed floor 3.9 against 4.1).
+// 3.07 and 3.83.  The streamed kernel: 2.67 against 2.84 ms inlined at three
+// blocks.  The plain kernel is faster with it inlined at three blocks (ward matrix
+// 8.1 against 8.6 ms).
 constexpr int kCallMinBlocks = 2;
 struct WedgeRest {
     uint32_t want, failed;

@@ -10,7 +10,8 @@ import torch
 
 import oracle
 import paper_2103_14137_gb300 as uvc
-from tests.gpu_util import T, build_arrays
+from synth.scenes import line_lamp, point_lamp
+from tests.gpu_util import T, build_arrays, lamp_of
 from tests.test_gpu_fluence import MU_TOL, _rel, _rows_of
 
 pytestmark = pytest.mark.gpu
@@ -55,4 +56,21 @@ def test_coverage_over_clusters(n, nvec):
     a = area.astype(np.float64)
     np.testing.assert_allclose(ca.cpu().numpy(), (ok * a).sum(1) / a.sum(), rtol=1e-6)
     np.testing.assert_allclose(cc.cpu().numpy(), ok.mean(1), rtol=1e-6)
+    sc.free()
+
+
+@pytest.mark.parametrize("nvec", [1, 31, 32, 33, 70])
+@pytest.mark.parametrize("nc", [1, 3, 19, 20, 21, 45])
+def test_streamed_stages_of_candidates_and_vectors(nc, nvec):
+    """Stages of 20 candidates by 32 vectors, whole and ragged, against the product of the stored entries: non-negative
+    sums of at most 45 terms in FP32, so within 50 x 2^-24 = 3e-6."""
+    rng, sc, _ = _points(100, nc + nvec)
+    cand = T(rng.uniform([0, 0, 1], [1, 1, 2], (nc, 3)).astype(np.float32))
+    t = rng.uniform(0, 60, size=(nvec, nc)).astype(np.float32)
+    t[:, ::4] = 0.0
+    for lamp in (lamp_of(point_lamp(80.0)), lamp_of(line_lamp(0.5, 3, 60.0))):
+        A, _ = uvc.irradiance_matrix(sc, cand, lamp)
+        ref = t.astype(np.float64) @ A[:, :100].cpu().numpy().astype(np.float64)
+        mu = uvc.fluence_streamed(sc, cand, lamp, T(t)).cpu().numpy()
+        assert _rel(mu, ref) <= 3e-6, _rel(mu, ref)
     sc.free()
