@@ -21,8 +21,11 @@
 namespace uvc {
 namespace {
 
-constexpr int kSortItems = 8;                      // keys per thread per tile
-constexpr int kSortTile = kThreads * kSortItems;   // 2048 keys per tile
+// Keys per thread of a tile of the sort: 8 where tiles of 2048 keys give every SM
+// one, 2 below that (a room of 30,000 triangles makes 15 tiles of 2048: a pass
+// took 18 us on 15 SMs).
+constexpr int kSortItemsMany = 8, kSortItemsFew = 2;
+constexpr int64_t kSortManyKeys = int64_t(152) * kThreads * kSortItemsMany;
 constexpr int kRadixBits = 8;
 constexpr int kRadixBins = 1 << kRadixBits;
 constexpr int kSortPasses = 8;                     // 64 bits of key
@@ -138,13 +141,15 @@ __global__ void k_morton(const float4* __restrict__ ref, int nt, const unsigned 
 }
 
 // Step 3a: per-tile digit histograms, laid out [digit][tile].
+template <int ITEMS>
 __global__ void __launch_bounds__(kThreads) k_radix_hist(const uint64_t* __restrict__ keys, int n, int shift,
                                                          int ntiles, uint32_t* __restrict__ hist) {
     __shared__ uint32_t h[kRadixBins];
     for (int d = threadIdx.x; d < kRadixBins; d += blockDim.x) h[d] = 0;
     __syncthreads();
-    int base = blockIdx.x * kSortTile;
-    for (int k = 0; k < kSortItems; ++k) {
+    int base = blockIdx.x * (kThreads * ITEMS);
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
         int idx = base + k * kThreads + threadIdx.x;
         if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & (kRadixBins - 1)], 1u);
     }
@@ -191,6 +196,7 @@ __global__ void __launch_bounds__(1024) k_radix_rowscan(uint32_t* __restrict__ h
 
 // Step 3c: stable scatter.  Within a tile, keys are ranked in index order
 // (warp chunk, then iteration, then lane) using warp match masks.
+template <int ITEMS>
 __global__ void __launch_bounds__(kThreads) k_radix_scatter(const uint64_t* __restrict__ keys_in,
                                                             const uint32_t* __restrict__ vals_in,
                                                             uint64_t* __restrict__ keys_out,
@@ -219,10 +225,10 @@ __global__ void __launch_bounds__(kThreads) k_radix_scatter(const uint64_t* __re
     for (int d = lane; d < kRadixBins; d += 32) cnt[warp][d] = 0;
     __syncthreads();
     const uint32_t lt = (1u << lane) - 1u;
-    const int base = blockIdx.x * kSortTile + warp * (32 * kSortItems);
-    uint64_t key[kSortItems];
-    uint32_t val[kSortItems], rank[kSortItems], dig[kSortItems];
-    for (int k = 0; k < kSortItems; ++k) {
+    const int base = blockIdx.x * (kThreads * ITEMS) + warp * (32 * ITEMS);
+    uint64_t key[ITEMS];
+    uint32_t val[ITEMS], rank[ITEMS], dig[ITEMS];
+    for (int k = 0; k < ITEMS; ++k) {
         int idx = base + k * 32 + lane;
         bool ok = idx < n;
         key[k] = ok ? keys_in[idx] : 0ull;
@@ -247,7 +253,7 @@ __global__ void __launch_bounds__(kThreads) k_radix_scatter(const uint64_t* __re
         }
     }
     __syncthreads();
-    for (int k = 0; k < kSortItems; ++k) {
+    for (int k = 0; k < ITEMS; ++k) {
         int idx = base + k * 32 + lane;
         if (idx >= n) continue;
         uint32_t d = dig[k];
@@ -573,13 +579,9 @@ __device__ __forceinline__ float box_half_area(const float* lo, const float* hi)
     return dx * dy + dy * dz + dz * dx;
 }
 
-__global__ void k_collapse_level(const Node* __restrict__ nodes, const int* __restrict__ fin,
-                                 const int* __restrict__ nin, int* __restrict__ fout, int* __restrict__ nout,
-                                 const int* __restrict__ leaf_loose, const int* __restrict__ node_loose,
-                                 Node4* __restrict__ nodes4) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= *nin) return;
-    const int i = fin[k];
+__device__ __forceinline__ void collapse_node(const Node* __restrict__ nodes, int i, int* fout, int* nout,
+                                              const int* __restrict__ leaf_loose, const int* __restrict__ node_loose,
+                                              Node4* __restrict__ nodes4) {
     int ref[4];
     float lo[4][3], hi[4][3];
     int cnt = 0;
@@ -633,6 +635,34 @@ __global__ void k_collapse_level(const Node* __restrict__ nodes, const int* __re
         int at = atomicAdd(nout, ninner);
         for (int c = 0; c < 4; ++c)
             if ((innermask >> c) & 1) fout[at++] = ref[c];
+    }
+}
+
+__global__ void k_collapse_level(const Node* __restrict__ nodes, const int* __restrict__ fin,
+                                 const int* __restrict__ nin, int* __restrict__ fout, int* __restrict__ nout,
+                                 const int* __restrict__ leaf_loose, const int* __restrict__ node_loose,
+                                 Node4* __restrict__ nodes4) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= *nin) return;
+    collapse_node(nodes, fin[k], fout, nout, leaf_loose, node_loose, nodes4);
+}
+
+// Levels L0 to L1 - 1 in one block, for the levels at both ends of the tree that
+// hold few nodes (a launch each cost more than the work: 22 launches of a room of
+// 30,000 triangles took 120 us).  Frontiers and counters are read past L1: the
+// block itself wrote them.
+__global__ void __launch_bounds__(1024) k_collapse_levels(const Node* __restrict__ nodes, int* fa, int* fb, int* counters,
+                                                          int L0, int L1, const int* __restrict__ leaf_loose,
+                                                          const int* __restrict__ node_loose,
+                                                          Node4* __restrict__ nodes4) {
+    for (int L = L0; L < L1; ++L) {
+        const int count = __ldcg(counters + L);
+        if (count == 0) return;
+        const int* fin = L & 1 ? fb : fa;
+        for (int k = threadIdx.x; k < count; k += blockDim.x)
+            collapse_node(nodes, __ldcg(fin + k), L & 1 ? fa : fb, counters + L + 1, leaf_loose, node_loose, nodes4);
+        __threadfence();
+        __syncthreads();
     }
 }
 
@@ -1029,7 +1059,9 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
 
     // temporaries
     const bool plates = !(flags_in & UVC_BUILD_LBVH_ONLY) && n > 1 && nt <= kPlateMaxTris;
-    const int ntiles = (n + kSortTile - 1) / kSortTile;
+    const bool few = n < kSortManyKeys;
+    const int tile = kThreads * (few ? kSortItemsFew : kSortItemsMany);
+    const int ntiles = (n + tile - 1) / tile;
     size_t tbytes = 3 * align256(sizeof(float4) * (size_t)n) +            // tri_lo, tri_hi, ref
                     align256(sizeof(uint64_t) * (size_t)n) +                // keys alt
                     2 * align256(sizeof(uint32_t) * (size_t)n) +            // vals, vals alt
@@ -1101,9 +1133,11 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
         uint32_t* vout = vals_alt;
         for (int pass = 0; pass < kSortPasses; ++pass) {
             int shift = pass * kRadixBits;
-            k_radix_hist<<<ntiles, kThreads, 0, stream>>>(kin, n, shift, ntiles, hist);
+            (few ? k_radix_hist<kSortItemsFew> : k_radix_hist<kSortItemsMany>)<<<ntiles, kThreads, 0, stream>>>(
+                kin, n, shift, ntiles, hist);
             k_radix_rowscan<<<kRadixBins, 1024, 0, stream>>>(hist, ntiles, totals);
-            k_radix_scatter<<<ntiles, kThreads, 0, stream>>>(kin, vin, kout, vout, n, shift, ntiles, hist, totals);
+            (few ? k_radix_scatter<kSortItemsFew> : k_radix_scatter<kSortItemsMany>)<<<ntiles, kThreads, 0, stream>>>(
+                kin, vin, kout, vout, n, shift, ntiles, hist, totals);
             uint64_t* tk = kin; kin = kout; kout = tk;
             uint32_t* tv = vin; vin = vout; vout = tv;
         }
@@ -1175,12 +1209,21 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
         int* counters = level_counts;   // depth + 2 <= n + 1 counters
         const int nlev = sc->depth + 1;
         k_collapse_start<<<(nlev + 1 + B - 1) / B, B, 0, stream>>>(fa, counters, nlev + 1);
-        for (int L = 0; L < nlev; ++L) {
+        // one block for the top (at most 4^4 nodes a level) and from four times the
+        // depth-balanced tree's nodes on, where few are left
+        int tail = 5;
+        while (tail < nlev && (tail >= 15 || (int64_t(1) << (2 * tail)) < 16 * (int64_t)n)) ++tail;
+        const int top = std::min(5, nlev);
+        k_collapse_levels<<<1, 1024, 0, stream>>>(sc->nodes, fa, fb, counters, 0, top, leaf_loose, node_loose, sc->nodes4);
+        for (int L = top; L < tail; ++L) {
             const int64_t bound = L < 15 ? std::min<int64_t>(ni, int64_t(1) << (2 * L)) : ni;
             k_collapse_level<<<(int)((bound + B - 1) / B), B, 0, stream>>>(sc->nodes, L & 1 ? fb : fa, counters + L,
                                                                          L & 1 ? fa : fb, counters + L + 1,
                                                                          leaf_loose, node_loose, sc->nodes4);
         }
+        if (tail < nlev)
+            k_collapse_levels<<<1, 1024, 0, stream>>>(sc->nodes, fa, fb, counters, tail, nlev, leaf_loose, node_loose,
+                                                      sc->nodes4);
         if (cudaGetLastError() != cudaSuccess) return fail(UVC_E_CUDA);
     }
     float diam = 0.f;
