@@ -74,3 +74,30 @@ def test_streamed_stages_of_candidates_and_vectors(nc, nvec):
         mu = uvc.fluence_streamed(sc, cand, lamp, T(t)).cpu().numpy()
         assert _rel(mu, ref) <= 3e-6, _rel(mu, ref)
     sc.free()
+
+
+@pytest.mark.parametrize("n", [1, 1023, 1025, 9000, 70001])
+def test_area_sums_keep_their_order(n):
+    """Coverage and the scene's area: 1024 compensated chains, then trees of 32 and 32, bit for bit."""
+    rng, sc, area = _points(n, n)
+    mu = rng.uniform(0, 2, (2, n)).astype(np.float32)
+
+    def total(a):   # masked patches leave their chain as it is
+        a = np.concatenate([a, np.full(-n % 1024, np.nan, np.float32)]).reshape(-1, 1024)
+        s, c = np.zeros(1024, np.float32), np.zeros(1024, np.float32)
+        for row in a:
+            ok = ~np.isnan(row)
+            y = row - c
+            t = s + y
+            c, s = np.where(ok, (t - s) - y, c), np.where(ok, t, s)
+        s = (s - c).reshape(32, 32)
+        for w in (16, 8, 4, 2, 1):
+            s = s[:, :w] + s[:, w:2 * w]
+        s = s[:, 0]
+        for w in (16, 8, 4, 2, 1):
+            s = s[:w] + s[w:2 * w]
+        return s[0]
+
+    got = uvc.coverage(sc, T(mu), 1.0)[0].cpu().numpy()
+    assert np.array_equal(got, np.float32([total(np.where(m >= 1.0, area, np.nan)) / total(area) for m in mu]))
+    sc.free()
