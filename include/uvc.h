@@ -162,8 +162,14 @@ int uvc_set_fluence_tensor_cores(int32_t enable, int32_t* previous);
  * every source is searched on its own.  Both give the visibility of Eq. (7)
  * source by source with the same segment test; they can differ only where a
  * segment grazes a triangle lying in the patch's own plane.  Scenes of more
- * than 2^27 triangles are always searched source by source.  The setting is
- * read when a call (or uvc_batch_create) converts its lamp.
+ * than 2^27 triangles are always searched source by source.
+ * With 1, all lamps also decide segments at the scene's plates first (flat
+ * axis-parallel rectangles that the mesh tiles completely, found by
+ * uvc_build_scene); with 0 the hierarchy is searched for everything.  The
+ * results are the same: a plate decides only segments that pass its borders
+ * and its plane by more than the segment test's rounding, and the hierarchy
+ * is searched for the rest.  Scenes with lowered limits do not use plates.
+ * The setting is read when a call (or uvc_batch_create) converts its lamp.
  *   enable    0 or 1
  *   previous  HOST int32, may be NULL: receives the setting before the call
  * Returns UVC_OK, or UVC_E_INVAL (setting unchanged) for other values of enable.
@@ -206,6 +212,8 @@ int uvc_irradiance_matrix(const uvc_scene* scene, const float* cand, int64_t nc,
  *             [3] per-segment box tests, [4] per-segment triangle tests,
  *             [5] facing segments that needed a search, [6] per-lane wedge
  *             box tests, [7] per-lane wedge plane tests
+ * The counted search is the hierarchy's for every segment: the plain call
+ * decides most segments of a room at its plates and makes fewer.
  * A packet is one warp: 32 patches and one lamp source (Sec. IV-C: each
  * segment is one source-to-patch visibility query of Eq. (7)), or, for a
  * vertical line lamp on the wedge path, 32 patches and all K sources of one
@@ -258,9 +266,10 @@ int uvc_irradiance_area_mean(const uvc_scene* scene, const float* cand, int64_t 
  *   workspace   device scratch; uvc_raster_workspace_bytes(scene, lamp, R, b)
  *               bytes hold batches of b candidates (more bytes, larger
  *               batches; less than b = 1 needs is UVC_E_INVAL)
- * A software rasteriser (setup, prefix-sum balanced fragments, watertight
- * pixel-centre ray tests with a 64-bit atomicMin of (depth, id)); the flux is
- * summed in 2^-40 W fixed point, so results do not depend on thread order.
+ * A software rasteriser by tiles of 64 x 64 pixels (triangles binned per tile,
+ * the tile's depth buffer in shared memory, watertight pixel-centre ray tests,
+ * the least (depth, id) wins); the flux is summed in 2^-40 W fixed point, so
+ * results do not depend on thread order.
  * R in [1, 4096].  Enqueued on `stream` (the table copy is synchronous with
  * the host).  Errors: UVC_E_INVAL, UVC_E_CUDA.
  */
@@ -602,7 +611,8 @@ int uvc_probe_l2_read(const void* buf, size_t bytes, int32_t passes, uint32_t* s
  *              float q[6][4] (per child pair the x, y, z records
  *              (c0.lo, c1.lo, c0.hi, c1.hi)), int32 r[4] (child refs: >= 0
  *              node, < 0 leaf ~k, 0x7fffffff empty), int32 m[4] (leaf mask,
- *              node mask, 0, 0)
+ *              node mask, mask of children that hold a triangle of no plate
+ *              (0 in builds without plates), 0)
  *   tri        float[nt][3][4]: vertices (x, y, z, w) in sorted order, w of
  *              the first vertex the triangle's input index (int32 bits)
  *   patch_s    float[np][4]: sample point and area

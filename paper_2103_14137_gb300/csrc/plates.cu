@@ -2,7 +2,7 @@
 // (walls, floors, the faces of furniture), found when a scene is built.  A
 // room's few dozen plates hold most of its triangles, and one test decides
 // what a segment does at a whole plate, so the searches try the plates first
-// (plates.cuh) and enter the hierarchy only for what they leave open.
+// (traverse.cuh) and enter the hierarchy only for what they leave open.
 //
 // A plate is a set of triangles, connected by shared edges, that
 //   - lie in one plane x = p, y = p or z = p, exactly (vertex coordinates are
@@ -24,6 +24,7 @@
 //   stats    per set: bounding rectangle and triangle count
 //   check    unshared edges must lie on their set's border
 //   select   sets that pass and hold at least kPlateMinTris triangles
+//   order    the larger plates first, those on the bounds last
 //   mark     triangles outside every plate mark their ancestors in the
 //            hierarchy, so that a search may skip subtrees of plates only
 // All of it is linear in the triangles and latency-bound on rooms.
