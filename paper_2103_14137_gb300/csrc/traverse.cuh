@@ -505,6 +505,11 @@ __device__ __forceinline__ PlateLane no_plate_lane() { return PlateLane{false, -
 // parameter a search would look at, dmax the longest segment.  Takes the
 // blocked sources out of `want` and returns the open ones among the rest (the
 // others are clear of every plate).  Every lane of the warp calls it.
+// UVC_PLATE_LOOP: a file whose kernel leaves the instruction cache (the area mean)
+// defines it to keep the loops over the sources rolled.
+#ifndef UVC_PLATE_LOOP
+#define UVC_PLATE_LOOP
+#endif
 template <bool ENDS, class Z>
 __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, int K, float cx, float cy, float sz,
                                                   float gx, float gy, float zlo, float zhi, float lend, float dmax,
@@ -589,7 +594,7 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
                                 const float e0 = fmaf(mu, zlo - sz, -mz), e1 = fmaf(mu, zhi - sz, -mz);
                                 if (ENDS && fmaxf(-e1, e0) - hz > w) clear = want;
                                 else if (ENDS && inside && fmaxf(-e0, e1) - hz < -w) blocked = want;
-                                else for (int q = 0; q < K; ++q) {
+                                else UVC_PLATE_LOOP for (int q = 0; q < K; ++q) {
                                     const float tz = fabsf(fmaf(mu, zsrc(q) - sz, -mz)) - hz;
                                     if (tz > w) clear |= 1u << q;
                                     else if (inside && tz < -w) blocked |= 1u << q;
@@ -623,7 +628,7 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
                                 }
                             }
                             if (!done)
-                                for (int q = 0; q < K; ++q) {
+                                UVC_PLATE_LOOP for (int q = 0; q < K; ++q) {
                                     const float hm = zsrc(q) - lo.z, dz = hm - hs;
                                     if (fabsf(hm) >= far_off) {
                                         const float ig = rcp_approx(dz), lam = hm * ig;
