@@ -16,6 +16,7 @@
 #include <cstring>
 #include <new>
 
+#include "collapse_plan.h"
 #include "uvc_internal.cuh"
 
 namespace uvc {
@@ -1207,23 +1208,18 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
         int* fa = height;
         int* fb = flags;
         int* counters = level_counts;   // depth + 2 <= n + 1 counters
-        const int nlev = sc->depth + 1;
-        k_collapse_start<<<(nlev + 1 + B - 1) / B, B, 0, stream>>>(fa, counters, nlev + 1);
-        // one block for the top (at most 4^4 nodes a level) and from four times the
-        // depth-balanced tree's nodes on, where few are left
-        int tail = 5;
-        while (tail < nlev && (tail >= 15 || (int64_t(1) << (2 * tail)) < 16 * (int64_t)n)) ++tail;
-        const int top = std::min(5, nlev);
-        k_collapse_levels<<<1, 1024, 0, stream>>>(sc->nodes, fa, fb, counters, 0, top, leaf_loose, node_loose, sc->nodes4);
-        for (int L = top; L < tail; ++L) {
+        const CollapsePlan cp = collapse_plan(sc->depth, n);
+        k_collapse_start<<<(cp.counters + B - 1) / B, B, 0, stream>>>(fa, counters, cp.counters);
+        k_collapse_levels<<<1, 1024, 0, stream>>>(sc->nodes, fa, fb, counters, 0, cp.top, leaf_loose, node_loose, sc->nodes4);
+        for (int L = cp.top; L < cp.tail; ++L) {
             const int64_t bound = L < 15 ? std::min<int64_t>(ni, int64_t(1) << (2 * L)) : ni;
             k_collapse_level<<<(int)((bound + B - 1) / B), B, 0, stream>>>(sc->nodes, L & 1 ? fb : fa, counters + L,
                                                                          L & 1 ? fa : fb, counters + L + 1,
                                                                          leaf_loose, node_loose, sc->nodes4);
         }
-        if (tail < nlev)
-            k_collapse_levels<<<1, 1024, 0, stream>>>(sc->nodes, fa, fb, counters, tail, nlev, leaf_loose, node_loose,
-                                                      sc->nodes4);
+        if (cp.tail < cp.levels)
+            k_collapse_levels<<<1, 1024, 0, stream>>>(sc->nodes, fa, fb, counters, cp.tail, cp.levels, leaf_loose,
+                                                      node_loose, sc->nodes4);
         if (cudaGetLastError() != cudaSuccess) return fail(UVC_E_CUDA);
     }
     float diam = 0.f;
