@@ -413,6 +413,12 @@ __global__ void k_node_depth(int n, const int* __restrict__ parent_int, const in
 // visits by 3 % (74.0 ms).
 constexpr int kTreelet = 5;
 constexpr int kRestructurePasses = 2;
+// Triangles up to which a warp restructures a treelet, a thread above: the warp has
+// the shorter chain up the tree, the thread the fewer instructions, and a large
+// mesh is bound by those.  Warp | thread, a whole build: 300,000 triangles 2.30 |
+// 2.38 ms (even), 2.59 | 2.84 (half of them in one place); 500,000 3.37 | 3.29, 3.67 |
+// 3.41; 2,000,000 11.3 | 9.7, 12.0 | 9.2; a floor of rooms (531,284) 4.48 | 3.97.
+constexpr int kWarpTreelets = 400000;
 constexpr float kCostNode = 1.2f, kCostTri = 1.0f;
 
 __device__ __forceinline__ float half_area(float4 lo, float4 hi) {
@@ -566,6 +572,128 @@ __global__ void __launch_bounds__(256) k_restructure(int n, TreeView T, const in
         restructure_treelet(T, p, lane);
         if (p == 0) return;
         p = __ldcg(&T.parent_int[p]);
+    }
+}
+
+// The same by one thread per treelet, a thread per leaf climbing: the working set in
+// local memory.
+__device__ void restructure_treelet_alone(const TreeView& T, int root) {
+    int tl[kTreelet];          // treelet leaves (refs)
+    int ti[kTreelet - 1];      // treelet internal nodes (reused)
+    const int2 rc = __ldcg(&T.children[root]);
+    tl[0] = rc.x;
+    tl[1] = rc.y;
+    int nl = 2, nin = 1;
+    ti[0] = root;
+    while (nl < kTreelet) {
+        int best = -1;
+        float best_a = -1.f;
+        for (int q = 0; q < nl; ++q) {
+            if (tl[q] < 0) continue;
+            float4 lo, hi;
+            ref_box(T, tl[q], lo, hi);
+            const float a = half_area(lo, hi);
+            if (a > best_a) { best_a = a; best = q; }
+        }
+        if (best < 0) break;
+        const int q = tl[best];
+        const int2 c = __ldcg(&T.children[q]);
+        ti[nin++] = q;
+        tl[best] = c.x;
+        tl[nl++] = c.y;
+    }
+    const float4 rlo = __ldcg(&T.node_lo[root]), rhi = __ldcg(&T.node_hi[root]);
+    // current cost of the root's subtree (children are final)
+    const float cur = kCostNode * half_area(rlo, rhi) + ref_cost(T, rc.x) + ref_cost(T, rc.y);
+    if (nl <= 2) {
+        __stcg(&T.cost[root], cur);
+        return;
+    }
+    const int nsub = 1 << nl;
+    float4 llo[kTreelet], lhi[kTreelet];
+    float copt[1 << kTreelet];
+    unsigned char part[1 << kTreelet];
+    for (int q = 0; q < nl; ++q) {
+        ref_box(T, tl[q], llo[q], lhi[q]);
+        copt[1 << q] = ref_cost(T, tl[q]);
+    }
+    auto set_box = [&](int S, float4& lo, float4& hi) {
+        lo = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
+        hi = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
+        for (int q = 0; q < nl; ++q)
+            if (S & (1 << q)) {
+                lo = make_float4(fminf(lo.x, llo[q].x), fminf(lo.y, llo[q].y), fminf(lo.z, llo[q].z), 0.f);
+                hi = make_float4(fmaxf(hi.x, lhi[q].x), fmaxf(hi.y, lhi[q].y), fmaxf(hi.z, lhi[q].z), 0.f);
+            }
+    };
+    for (int S = 1; S < nsub; ++S) {
+        const int low = S & -S;
+        if (S == low) continue;
+        float best = 3.0e38f;
+        int bp = low;
+        // partitions (P, S\P) with P holding S's lowest leaf
+        for (int P = (S - 1) & S; P != 0; P = (P - 1) & S) {
+            if (!(P & low)) continue;
+            const float c = copt[P] + copt[S ^ P];
+            if (c < best) { best = c; bp = P; }
+        }
+        float4 lo, hi;
+        set_box(S, lo, hi);
+        copt[S] = kCostNode * half_area(lo, hi) + best;
+        part[S] = (unsigned char)bp;
+    }
+    const int full = nsub - 1;
+    if (!(copt[full] < cur * 0.999f)) {
+        __stcg(&T.cost[root], cur);
+        return;
+    }
+    // rewire: the root keeps its index and parent; other internal nodes are reused
+    int st_set[kTreelet], st_node[kTreelet];
+    int top = 0, next = 1;
+    st_set[top] = full;
+    st_node[top] = root;
+    ++top;
+    while (top > 0) {
+        --top;
+        const int S = st_set[top], node = st_node[top];
+        const int P = part[S], Q = S ^ P;
+        int ref[2];
+        const int sets[2] = {P, Q};
+        for (int h = 0; h < 2; ++h) {
+            const int X = sets[h];
+            if ((X & (X - 1)) == 0) {
+                ref[h] = tl[__ffs(X) - 1];
+            } else {
+                const int m = ti[next++];
+                ref[h] = m;
+                st_set[top] = X;
+                st_node[top] = m;
+                ++top;
+            }
+            if (ref[h] < 0) T.parent_leaf[~ref[h]] = node;
+            else T.parent_int[ref[h]] = node;
+        }
+        float4 lo, hi;
+        set_box(S, lo, hi);
+        __stcg(&T.children[node], make_int2(ref[0], ref[1]));
+        __stcg(&T.node_lo[node], lo);
+        __stcg(&T.node_hi[node], hi);
+        __stcg(&T.cost[node], copt[S]);
+    }
+}
+
+__global__ void k_restructure_alone(int n, TreeView T, const int* __restrict__ leaf_parent0, int* flags) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    int p = leaf_parent0[k];
+    while (p >= 0) {
+        __threadfence();
+        if (atomicAdd(&flags[p], 1) == 0) return;   // the sibling subtree finishes p
+        __threadfence();
+        restructure_treelet_alone(T, p);
+        __threadfence();
+        if (p == 0) return;
+        p = T.parent_int[p];
     }
 }
 
@@ -1164,7 +1292,10 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
                     cudaMemsetAsync(flags, 0, sizeof(int) * (size_t)ni, stream);
                     cudaMemcpyAsync(leaf_parent0, parent_leaf, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice,
                                     stream);
-                    k_restructure<<<(n + kWarpsPerBlock - 1) / kWarpsPerBlock, kThreads, 0, stream>>>(n, T, leaf_parent0, flags);
+                    if (n <= kWarpTreelets)
+                        k_restructure<<<(n + kWarpsPerBlock - 1) / kWarpsPerBlock, kThreads, 0, stream>>>(n, T, leaf_parent0, flags);
+                    else
+                        k_restructure_alone<<<(n + 127) / 128, 128, 0, stream>>>(n, T, leaf_parent0, flags);
                 }
             }
             if (plates) {
