@@ -1200,6 +1200,13 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
     const bool few = n < kSortManyKeys;
     const int tile = kThreads * (few ? kSortItemsFew : kSortItemsMany);
     const int ntiles = (n + tile - 1) / tile;
+    // The search for plates works in the arrays of the steps before it that nothing
+    // reads any more (the first twelve below).  A block of its own, 108 bytes a
+    // triangle, cost more to map than the search takes: 0.4 ms of a build of
+    // 2,000,000 triangles.
+    const size_t spent = sizeof(float4) * 3 * (size_t)n + sizeof(uint64_t) * (size_t)n + sizeof(uint32_t) * 2 * (size_t)n +
+                         sizeof(int) * ((size_t)n + 3 * (size_t)ni);
+    const size_t plates_need = plates ? plates_work_bytes(nt) : 0, plates_more = plates_need > spent ? plates_need - spent : 0;
     size_t tbytes = 3 * align256(sizeof(float4) * (size_t)n) +            // tri_lo, tri_hi, ref
                     align256(sizeof(uint64_t) * (size_t)n) +                // keys alt
                     2 * align256(sizeof(uint32_t) * (size_t)n) +            // vals, vals alt
@@ -1213,7 +1220,7 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
                     align256(sizeof(int) * (size_t)n) +                      // leaf parents at pass start
                     align256(sizeof(unsigned int) * 12) + align256(sizeof(int) * 4) +
                     align256(sizeof(int) * (size_t)n) + align256(sizeof(int) * (size_t)ni) +   // loose leaves, nodes
-                    (plates ? align256(plates_work_bytes(nt)) : 0) +
+                    align256(plates_more) +
                     align256(sizeof(int) * ((size_t)n + 2)) + 256;                    // collapse level counters
     void* tblock = nullptr;
     if (cudaMallocAsync(&tblock, tbytes, stream) != cudaSuccess) {
@@ -1231,6 +1238,12 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
     uint32_t* vals_alt = tc.take<uint32_t>(n);
     uint32_t* hist = tc.take<uint32_t>(kRadixBins * (size_t)ntiles);
     uint32_t* totals = tc.take<uint32_t>(kRadixBins);
+    int* height = tc.take<int>(ni);
+    int* ndepth = tc.take<int>(ni);
+    float* cost = tc.take<float>(ni);
+    int* leaf_parent0 = tc.take<int>(n);
+    if (plates_need > tc.off) tc.take<char>(plates_need - tc.off);   // at most plates_more
+    char* plates_work = static_cast<char*>(tblock);
     int2* children = tc.take<int2>(ni);
     int* parent_int = tc.take<int>(ni);
     int* parent_leaf = tc.take<int>(n);
@@ -1238,16 +1251,11 @@ int build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
     float4* leaf_hi = tc.take<float4>(n);
     float4* node_lo = tc.take<float4>(ni);
     float4* node_hi = tc.take<float4>(ni);
-    int* height = tc.take<int>(ni);
     int* flags = tc.take<int>(ni);
-    int* ndepth = tc.take<int>(ni);
-    float* cost = tc.take<float>(ni);
-    int* leaf_parent0 = tc.take<int>(n);
     unsigned int* bounds = tc.take<unsigned int>(12);   // reference points lo/hi, triangle boxes lo/hi
     int* errdepth = tc.take<int>(5);   // [0] = error bits, [1] = depth, [2] = plates, [3] = loose triangles, [4] = inner plates' triangles
     int* leaf_loose = tc.take<int>(n);
     int* node_loose = tc.take<int>(ni);
-    char* plates_work = plates ? tc.take<char>(plates_work_bytes(nt)) : nullptr;
     int* level_counts = tc.take<int>((size_t)n + 2);   // four-wide nodes per level of the collapse
 
     cudaError_t e = cudaSuccess;

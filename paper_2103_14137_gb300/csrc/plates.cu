@@ -27,6 +27,7 @@
 //   order    the larger plates first, those on the bounds last
 //   mark     triangles outside every plate mark their ancestors in the
 //            hierarchy, so that a search may skip subtrees of plates only
+//            (none where there are no plates)
 // All of it is linear in the triangles and latency-bound on rooms.
 #include "uvc_internal.cuh"
 
@@ -106,13 +107,21 @@ __device__ __forceinline__ uint32_t edge_hash(const Flat& f, const Edge& g) {
 }
 
 // Root of x's set.  Parents only ever move to smaller indices, so the walk
-// ends; halving the path keeps it short.
+// ends; halving the path keeps it short.  Read through L1: an old parent is an
+// ancestor all the same, and an old root is found out by the exchange in set_join
+// (the floor of a floor of rooms is one set of some 80,000 triangles; with all of
+// them reading its root from one L2 line k_plate_edges took 427 us there, now 294).
+__device__ __forceinline__ int parent_of(const int* parent, int x) {
+    int q;
+    asm volatile("ld.global.ca.s32 %0, [%1];" : "=r"(q) : "l"(parent + x) : "memory");
+    return q;
+}
+
 __device__ __forceinline__ int set_root(int* parent, int x) {
-    volatile int* p = parent;
-    int q = p[x];
+    int q = parent_of(parent, x);
     while (q != x) {
-        const int g = p[q];
-        if (g != q) p[x] = g;
+        const int g = parent_of(parent, q);
+        if (g != q) parent[x] = g;
         x = q;
         q = g;
     }
@@ -120,12 +129,13 @@ __device__ __forceinline__ int set_root(int* parent, int x) {
 }
 
 __device__ __forceinline__ void set_join(int* parent, int a, int b) {
-    for (;;) {   // each failed exchange means that another thread lowered parent[a]
-        a = set_root(parent, a);
-        b = set_root(parent, b);
-        if (a == b) return;
+    a = set_root(parent, a);
+    b = set_root(parent, b);
+    while (a != b) {   // each failed exchange gives a parent below a
         if (a < b) { const int t = a; a = b; b = t; }
-        if (atomicCAS(&parent[a], a, b) == a) return;
+        const int now = atomicCAS(&parent[a], a, b);
+        if (now == a) return;
+        a = set_root(parent, now);
     }
 }
 
@@ -137,27 +147,28 @@ __global__ void k_plate_init(const float4* __restrict__ tri, int nt, int* __rest
     state[k] = 0u;
 }
 
-constexpr unsigned kStateBad = 8u;   // state: bit e = edge e has its mate, kStateBad = an edge is shared wrongly
+// state: bit e = edge e has its mate, kStateBad = an edge is shared wrongly, bit
+// 4 + e = edge e is in the table and has been taken by a mate
+constexpr unsigned kStateBad = 8u, kStateTaken = 16u;
 
-__global__ void k_plate_edges(const float4* __restrict__ tri, int nt, int2* __restrict__ table, uint32_t mask,
+__global__ void k_plate_edges(const float4* __restrict__ tri, int nt, int* __restrict__ table, uint32_t mask,
                               int* __restrict__ parent, unsigned* __restrict__ state) {
     const int id = blockIdx.x * blockDim.x + threadIdx.x;   // 4 k + e
     const int k = id >> 2, e = id & 3;
-    if (k >= nt || e == 3) return;
+    if (k >= nt || e == 3 || parent_of(parent, k) < 0) return;
     const Flat f = flat_of(tri, k);
-    if (f.axis < 0) return;
     const Edge g = edge_of(f, e);
     uint32_t h = edge_hash(f, g) & mask;
     for (int probe = 0; probe < kMaxProbes; ++probe, h = (h + 1) & mask) {
-        int* slot = reinterpret_cast<int*>(table + h);
-        int own = *reinterpret_cast<volatile int*>(slot);
-        if (own == -1) own = atomicCAS(slot, -1, id);
+        int own = *reinterpret_cast<volatile int*>(table + h);
+        if (own == -1) own = atomicCAS(table + h, -1, id);
         if (own == -1) return;   // first of its kind
         const Flat o = flat_of(tri, own >> 2);
         if (o.axis != f.axis || o.ccw != f.ccw || o.p != f.p) continue;
         const Edge q = edge_of(o, own & 3);
         if (q.u0 != g.u0 || q.v0 != g.v0 || q.u1 != g.u1 || q.v1 != g.v1) continue;
-        if (q.up != g.up && atomicCAS(slot + 1, -1, id) == -1) {
+        const unsigned taken = kStateTaken << (own & 3);
+        if (q.up != g.up && !(atomicOr(&state[own >> 2], taken) & taken)) {
             atomicOr(&state[k], 1u << e);
             atomicOr(&state[own >> 2], 1u << (own & 3));
             set_join(parent, k, own >> 2);
@@ -319,8 +330,13 @@ __global__ void k_plate_mark(const float4* __restrict__ tri, int nt, int* __rest
                              const int* __restrict__ plate_id, const int* __restrict__ place_of,
                              const int* __restrict__ parent_leaf,
                              const int* __restrict__ parent_int, int2* __restrict__ place,
-                             int* __restrict__ leaf_loose, int* __restrict__ node_loose, int* __restrict__ nloose) {
+                             int* __restrict__ leaf_loose, int* __restrict__ node_loose, const int* __restrict__ nplate,
+                             int* __restrict__ nloose) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (*nplate == 0) {   // nothing to look up or to skip: no marks, and the places are not read
+        if (k < nt) leaf_loose[k] = 0;
+        return;
+    }
     int plate = 0;
     if (k < nt) {
         plate = parent[k] >= 0 ? plate_id[set_root(parent, k)] : -1;
@@ -340,7 +356,8 @@ __global__ void k_plate_mark(const float4* __restrict__ tri, int nt, int* __rest
 // decides, which knows the excluded triangles).
 __global__ void k_plate_patches(const float4* __restrict__ ps, const int2* __restrict__ pe, int np, int nt,
                                 const int2* __restrict__ place, const float4* __restrict__ plates,
-                                uint32_t* __restrict__ flags) {
+                                const int* __restrict__ nplate, uint32_t* __restrict__ flags) {
+    if (*nplate == 0) return;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     bool flag = false;
     if (j < np) {
@@ -372,7 +389,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Bytes of find_plates' workspace.
 size_t plates_work_bytes(int64_t nt) {
-    return align256(sizeof(int2) * (size_t)table_slots(nt)) + 5 * align256(sizeof(int) * (size_t)nt) +
+    return align256(sizeof(int) * (size_t)table_slots(nt)) + 5 * align256(sizeof(int) * (size_t)nt) +
            3 * align256(sizeof(int2) * (size_t)nt) + align256(sizeof(int) * kMaxPlates);
 }
 
@@ -388,7 +405,7 @@ void find_plates(uvc_scene* sc, const int* parent_leaf, const int* parent_int, i
     const uint32_t slots = table_slots(nt);
     char* p = static_cast<char*>(work);
     auto take = [&](size_t n) { char* q = p; p += align256(n); return q; };
-    int2* table = reinterpret_cast<int2*>(take(sizeof(int2) * (size_t)slots));
+    int* table = reinterpret_cast<int*>(take(sizeof(int) * (size_t)slots));
     int* parent = reinterpret_cast<int*>(take(sizeof(int) * (size_t)nt));
     unsigned* state = reinterpret_cast<unsigned*>(take(sizeof(int) * (size_t)nt));
     int* plate_id = reinterpret_cast<int*>(take(sizeof(int) * (size_t)nt));
@@ -398,7 +415,7 @@ void find_plates(uvc_scene* sc, const int* parent_leaf, const int* parent_int, i
     unsigned* len = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * (size_t)nt));
     float* area2 = reinterpret_cast<float*>(take(sizeof(float) * (size_t)nt));
     int* place_of = reinterpret_cast<int*>(take(sizeof(int) * kMaxPlates));
-    cudaMemsetAsync(table, 0xff, sizeof(int2) * (size_t)slots, stream);
+    cudaMemsetAsync(table, 0xff, sizeof(int) * (size_t)slots, stream);
     cudaMemsetAsync(lo, 0xff, sizeof(uint2) * (size_t)nt, stream);
     cudaMemsetAsync(hi, 0, (char*)(area2 + nt) - (char*)hi, stream);   // hi, cnt_bad, len, area2
     k_plate_init<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, state);
@@ -409,9 +426,9 @@ void find_plates(uvc_scene* sc, const int* parent_leaf, const int* parent_int, i
                                                  box, counts, counts + 2);
     k_plate_order<<<1, kMaxPlates, 0, stream>>>(sc->plates, counts, box, place_of);
     k_plate_mark<<<grid(nt), 256, 0, stream>>>(sc->tri, nt, parent, plate_id, place_of, parent_leaf, parent_int, sc->tri_place,
-                                               leaf_loose, node_loose, counts + 1);
+                                               leaf_loose, node_loose, counts, counts + 1);
     if (np > 0)
-        k_plate_patches<<<grid(np), 256, 0, stream>>>(sc->patch_s, sc->patch_excl, np, nt, sc->tri_place, sc->plates,
+        k_plate_patches<<<grid(np), 256, 0, stream>>>(sc->patch_s, sc->patch_excl, np, nt, sc->tri_place, sc->plates, counts,
                                                       reinterpret_cast<uint32_t*>(sc->plates + 2 * kMaxPlates));
 }
 
