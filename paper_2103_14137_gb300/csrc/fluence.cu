@@ -80,8 +80,9 @@ __global__ void __launch_bounds__(256, 2) k_fluence(const float* __restrict__ A,
         // permuted by the row so that the lanes' stores (consecutive rows) meet 8
         // banks and not 2
         float* tsf = reinterpret_cast<float*>(ts);
-        for (int e = gt; e < kFlChunk * kNV; e += kFlGroupThreads) {
-            const int v = e / kFlChunk, q = e % kFlChunk;
+        const int lg = c1 - c0 > 64 ? 7 : (c1 - c0 > 32 ? 6 : 5);   // 2^lg rows, of 128: a short matrix has no more
+        for (int e = gt; c1 > c0 && e < kNV << lg; e += kFlGroupThreads) {
+            const int v = e >> lg, q = e & ((1 << lg) - 1);
             const int i = c0 + q;
             tsf[q * kNV + ((v >> 2) ^ ((q >> 1) & 3)) * 4 + (v & 3)] = (i < c1 && v0 + v < nvec) ? __ldg(&t[(size_t)(v0 + v) * nc + i]) : 0.f;
         }
@@ -154,11 +155,106 @@ __global__ void __launch_bounds__(256, 2) k_fluence(const float* __restrict__ A,
     cluster.sync();   // no block leaves while its results are read
 }
 
+// k_fluence_wide: matrices of more columns than the clusters are for, whose rows
+// allow no tensor map.  One block per 128 columns and 16 vectors, a thread two
+// columns and all 16 vectors, so each value of A is read once; sums in the order of
+// k_fluence with one block a cluster (the same bits).  98,132 columns, 2,000 rows, 16
+// vectors in an odd row length: 439 us, with k_fluence 648.
+constexpr int kFwUnroll = 4;                      // rows of A loaded ahead
+__global__ void __launch_bounds__(256, 2) k_fluence_wide(const float* __restrict__ A, int nc, int64_t lda,
+                                                         const float* __restrict__ t, int nvec, int v0,
+                                                         float* __restrict__ mu, int np, int vec2) {
+    extern __shared__ float4 fluence_smem[];
+    const int g = threadIdx.x / kFlGroupThreads, gt = threadIdx.x % kFlGroupThreads;
+    float4* ts = fluence_smem + (size_t)g * kFlChunk * (kNV / 4);   // [kFlChunk][kNV / 4]
+    const int j0 = blockIdx.x * kFlCols + 2 * gt;
+    const bool ok0 = j0 < np, ok1 = j0 + 1 < np;
+    const int per = (((nc + kFlGroups - 1) / kFlGroups) + 31) / 32 * 32;   // rows per group, multiple of 32
+    const int r0 = min(nc, g * per), r1 = min(nc, r0 + per);
+    float2 part[kNV], acc[kNV], comp[kNV];
+#pragma unroll
+    for (int v = 0; v < kNV; ++v) {
+        part[v] = make_float2(0.f, 0.f);
+        acc[v] = part[v];
+        comp[v] = part[v];
+    }
+    const int nchunk = (per + kFlChunk - 1) / kFlChunk;   // the same for every group
+    for (int ck = 0; ck < nchunk; ++ck) {
+        const int c0 = r0 + ck * kFlChunk, c1 = min(r1, c0 + kFlChunk);
+        __syncthreads();
+        // stage t[v0 + v][c0 .. c1) transposed: ts[row][v]
+        float* tsf = reinterpret_cast<float*>(ts);
+        for (int e = gt; e < kFlChunk * kNV; e += kFlGroupThreads) {
+            const int v = e / kFlChunk, q = e % kFlChunk;
+            const int i = c0 + q;
+            tsf[q * kNV + v] = (i < c1 && v0 + v < nvec) ? __ldg(&t[(size_t)(v0 + v) * nc + i]) : 0.f;
+        }
+        __syncthreads();
+        for (int q0 = 0; q0 < c1 - c0; q0 += kFwUnroll) {
+            float2 a[kFwUnroll];
+#pragma unroll
+            for (int u = 0; u < kFwUnroll; ++u) {
+                const int i = c0 + q0 + u;
+                a[u] = make_float2(0.f, 0.f);
+                if (i < c1) {
+                    const float* row = A + (size_t)i * lda + j0;
+                    if (vec2 && ok1) {
+                        a[u] = __ldcs(reinterpret_cast<const float2*>(row));
+                    } else {
+                        if (ok0) a[u].x = __ldcs(row);
+                        if (ok1) a[u].y = __ldcs(row + 1);
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kFwUnroll; ++u) {
+#pragma unroll
+                for (int v4 = 0; v4 < kNV / 4; ++v4) {
+                    const float4 w = ts[(q0 + u) * (kNV / 4) + v4];   // rows past c1 hold zeros
+                    part[4 * v4 + 0] = __ffma2_rn(make_float2(w.x, w.x), a[u], part[4 * v4 + 0]);
+                    part[4 * v4 + 1] = __ffma2_rn(make_float2(w.y, w.y), a[u], part[4 * v4 + 1]);
+                    part[4 * v4 + 2] = __ffma2_rn(make_float2(w.z, w.z), a[u], part[4 * v4 + 2]);
+                    part[4 * v4 + 3] = __ffma2_rn(make_float2(w.w, w.w), a[u], part[4 * v4 + 3]);
+                }
+            }
+            if (((q0 + kFwUnroll) & 31) == 0 || q0 + kFwUnroll >= c1 - c0) {   // a block of 32 rows ends
+#pragma unroll
+                for (int v = 0; v < kNV; ++v) {
+                    kahan_add(acc[v].x, comp[v].x, part[v].x);
+                    kahan_add(acc[v].y, comp[v].y, part[v].y);
+                    part[v] = make_float2(0.f, 0.f);
+                }
+            }
+        }
+    }
+    // fixed-order (group 0..3) compensated sum of the group results
+    __syncthreads();
+    float2* red = reinterpret_cast<float2*>(fluence_smem);   // [kFlGroups][kNV][kFlGroupThreads]
+#pragma unroll
+    for (int v = 0; v < kNV; ++v)
+        red[((size_t)g * kNV + v) * kFlGroupThreads + gt] =
+            make_float2(__fsub_rn(acc[v].x, comp[v].x), __fsub_rn(acc[v].y, comp[v].y));
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < kNV * kFlGroupThreads; idx += blockDim.x) {
+        const int v = idx / kFlGroupThreads, l = idx % kFlGroupThreads;
+        const int jj = blockIdx.x * kFlCols + 2 * l;
+        if (v0 + v >= nvec) continue;
+        float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
+        for (int w = 0; w < kFlGroups; ++w) {
+            const float2 x = red[((size_t)w * kNV + v) * kFlGroupThreads + l];
+            kahan_add(s0, c0, x.x);
+            kahan_add(s1, c1, x.y);
+        }
+        if (jj < np) mu[(size_t)(v0 + v) * np + jj] = s0;
+        if (jj + 1 < np) mu[(size_t)(v0 + v) * np + jj + 1] = s1;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Fluence with the rows of A fed by the tensor-memory accelerator
 // ---------------------------------------------------------------------------
-// The same block shape and summation order as k_fluence (so the same bits),
-// but A does not pass through registers: each row group streams its rows
+// The block shape and summation order of k_fluence_wide (so the same bits), but A
+// does not pass through registers: each row group streams its rows
 // through a ring of kTmaStages shared-memory tiles of kTmaRows x 128 floats,
 // loaded by cp.async.bulk.tensor (one 2-D tensor-map copy per tile, issued by
 // the group's first thread) and completed on an mbarrier per tile.  Up to
@@ -795,7 +891,7 @@ int fluence(const uvc_scene* sc, const float* A, int64_t nc, int64_t lda, const 
             k_fluence_tc<<<grid, kTcThreads, kTcSmem, stream>>>(map, (int)nc, t, nvec, v0, mu, np, sc->status);
         return status_from_cuda(cudaGetLastError());
     }
-    if (!narrow && S == 1 && fluence_tensor_map(A, nc, lda, np, kTmaRows, &map)) {
+    if (!narrow && fluence_tensor_map(A, nc, lda, np, kTmaRows, &map)) {
         static const cudaError_t tattr =
             cudaFuncSetAttribute(k_fluence_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTmaSmem);
         if (tattr != cudaSuccess) return status_from_cuda(tattr);
@@ -805,11 +901,17 @@ int fluence(const uvc_scene* sc, const float* A, int64_t nc, int64_t lda, const 
             k_fluence_tma<<<grid, kThreads, kTmaSmem, stream>>>(map, (int)nc, t, nvec, v0, mu, np, sc->status);
         return status_from_cuda(cudaGetLastError());
     }
+    const int vec2 = (lda % 2 == 0) && (reinterpret_cast<uintptr_t>(A) % 8 == 0);
+    if (!narrow) {
+        for (int v0 = 0; v0 < nvec; v0 += kNV)
+            k_fluence_wide<<<(np + kFlCols - 1) / kFlCols, kThreads, kFluenceSmem, stream>>>(A, (int)nc, lda, t, nvec, v0, mu,
+                                                                                             np, vec2);
+        return status_from_cuda(cudaGetLastError());
+    }
     // once per process (and so not during a stream capture that follows a first call)
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_fluence, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFluenceSmem);
     if (attr != cudaSuccess) return status_from_cuda(attr);
-    const int vec2 = (lda % 2 == 0) && (reinterpret_cast<uintptr_t>(A) % 8 == 0);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(cols * S), (unsigned)passes, 1);
     cfg.blockDim = dim3(256, 1, 1);
