@@ -728,30 +728,32 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_fluence_tc(const __grid_const
     }
 }
 
-// Sums over the patches by a cluster of kSumBlocks blocks: area sum and count of
-// the patches that `in` accepts; the result in thread 0 of rank 0.  The order of
-// the additions is fixed: 1024 compensated chains (patch j in chain j mod 1024),
-// a tree over each 32 of them and a tree over those (other orders move the
-// scene's area by an ulp, and every feature normalised by it).  One block read
-// 98,132 patches in 32 us (the areas) and 54-75 us (with 4 to 16 vectors).
-constexpr int kSumBlocks = 8, kSumThreads = 128, kSumAhead = 8;
-static_assert(kSumBlocks * kSumThreads == 1024, "one chain per thread");
-template <class In>
-__device__ __forceinline__ void cluster_sum(const float4* __restrict__ ps, int np, In in, float& s, unsigned long long& n) {
+// Sums over the patches: area sum and count of the patches that `in` accepts; the
+// result in thread 0 of rank 0.  The order of the additions is fixed: 1024
+// compensated chains (patch j in chain j mod 1024), a tree over each 32 of them and
+// a tree over those (other orders move the scene's area by an ulp, and every feature
+// normalised by it).  One block of 1024 threads, or a cluster of kSumBlocks that
+// shares out the chains: one block read 98,132 patches in 32 us (the areas) and
+// 54-75 us (with 4 to 16 vectors),
+// now one vector in 3 us more than a cluster; for 40,000 patches the block is as
+// fast and for 300 1 us faster, and with 256 vectors of 98,132 (45 | 51 us).
+constexpr int kSumBlocks = 8, kSumAhead = 8, kSumChains = 1024;
+template <int BLOCKS, class In>
+__device__ __forceinline__ void patch_sum(const float4* __restrict__ ps, int np, In in, float& s, unsigned long long& n) {
     namespace cg = cooperative_groups;
+    constexpr int kThreadsEach = kSumChains / BLOCKS;
     __shared__ float sum_of[32];
     __shared__ unsigned long long count_of[32];
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank(), step = kSumBlocks * kSumThreads;
+    const int rank = BLOCKS > 1 ? (int)cg::this_cluster().block_rank() : 0;
     float c = 0.f;
     s = 0.f;
     n = 0;
-    for (int64_t j0 = rank * kSumThreads + (int)threadIdx.x; j0 < np; j0 += (int64_t)kSumAhead * step) {
+    for (int64_t j0 = rank * kThreadsEach + (int)threadIdx.x; j0 < np; j0 += (int64_t)kSumAhead * kSumChains) {
         bool ok[kSumAhead];
         float a[kSumAhead];
 #pragma unroll
         for (int q = 0; q < kSumAhead; ++q) {
-            const int64_t j = j0 + (int64_t)q * step;
+            const int64_t j = j0 + (int64_t)q * kSumChains;
             ok[q] = j < np && in(j);
             a[q] = j < np ? __ldg(&ps[j].w) : 0.f;
         }
@@ -769,14 +771,23 @@ __device__ __forceinline__ void cluster_sum(const float4* __restrict__ ps, int n
             n += __shfl_down_sync(0xffffffffu, n, o);
         }
     };
-    const int lane = threadIdx.x & 31, warp = rank * (kSumThreads / 32) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, warp = rank * (kThreadsEach / 32) + (threadIdx.x >> 5);
     tree();
-    cluster.sync();   // rank 0 runs: its memory may be written
-    if (lane == 0) {
-        cluster.map_shared_rank(sum_of, 0)[warp] = s;
-        cluster.map_shared_rank(count_of, 0)[warp] = n;
+    if constexpr (BLOCKS > 1) {
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();   // rank 0 runs: its memory may be written
+        if (lane == 0) {
+            cluster.map_shared_rank(sum_of, 0)[warp] = s;
+            cluster.map_shared_rank(count_of, 0)[warp] = n;
+        }
+        cluster.sync();
+    } else {
+        if (lane == 0) {
+            sum_of[warp] = s;
+            count_of[warp] = n;
+        }
+        __syncthreads();
     }
-    cluster.sync();
     if (warp == 0) {
         s = sum_of[lane];
         n = count_of[lane];
@@ -784,34 +795,57 @@ __device__ __forceinline__ void cluster_sum(const float4* __restrict__ ps, int n
     }
 }
 
-__global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kSumThreads)
-    k_area_total(const float4* __restrict__ ps, int np, float* out) {
+template <int BLOCKS>
+__device__ __forceinline__ void area_total(const float4* __restrict__ ps, int np, float* out) {
     float s;
     unsigned long long n;
-    cluster_sum(ps, np, [](int64_t) { return true; }, s, n);
+    patch_sum<BLOCKS>(ps, np, [](int64_t) { return true; }, s, n);
     if (blockIdx.x == 0 && threadIdx.x == 0) *out = s;
 }
 
-// One cluster per dwell vector.
-__global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kSumThreads)
-    k_coverage(const float* __restrict__ mu, int np, float mu_min, const float4* __restrict__ ps,
-               const float* __restrict__ area_total, float* __restrict__ cov_area, float* __restrict__ cov_count) {
-    const int v = blockIdx.x / kSumBlocks;
+// One block or cluster per dwell vector.
+template <int BLOCKS>
+__device__ __forceinline__ void coverage_of(const float* __restrict__ mu, int np, float mu_min, const float4* __restrict__ ps,
+                                            const float* __restrict__ area_total, float* __restrict__ cov_area,
+                                            float* __restrict__ cov_count) {
+    const int v = blockIdx.x / BLOCKS;
     const float* m = mu + (size_t)v * np;
     float s;
     unsigned long long n;
-    cluster_sum(ps, np, [&](int64_t j) { return __ldg(m + j) >= mu_min; }, s, n);
-    if (blockIdx.x % kSumBlocks == 0 && threadIdx.x == 0) {
+    patch_sum<BLOCKS>(ps, np, [&](int64_t j) { return __ldg(m + j) >= mu_min; }, s, n);
+    if (blockIdx.x % BLOCKS == 0 && threadIdx.x == 0) {
         const float tot = *area_total;
         cov_area[v] = tot > 0.f ? __fdiv_rn(s, tot) : 0.f;
         if (cov_count) cov_count[v] = np > 0 ? __fdiv_rn((float)n, (float)np) : 0.f;
     }
 }
 
+__global__ void __launch_bounds__(kSumChains) k_area_total(const float4* __restrict__ ps, int np, float* out) {
+    area_total<1>(ps, np, out);
+}
+__global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kSumChains / kSumBlocks)
+    k_area_total_split(const float4* __restrict__ ps, int np, float* out) {
+    area_total<kSumBlocks>(ps, np, out);
+}
+__global__ void __launch_bounds__(kSumChains)
+    k_coverage(const float* __restrict__ mu, int np, float mu_min, const float4* __restrict__ ps,
+               const float* __restrict__ area_total, float* __restrict__ cov_area, float* __restrict__ cov_count) {
+    coverage_of<1>(mu, np, mu_min, ps, area_total, cov_area, cov_count);
+}
+__global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kSumChains / kSumBlocks)
+    k_coverage_split(const float* __restrict__ mu, int np, float mu_min, const float4* __restrict__ ps,
+                     const float* __restrict__ area_total, float* __restrict__ cov_area, float* __restrict__ cov_count) {
+    coverage_of<kSumBlocks>(mu, np, mu_min, ps, area_total, cov_area, cov_count);
+}
+
+// A cluster each where one block would read for long and `sums` of them leave SMs idle.
+bool split_sums(int64_t np, int64_t sums) { return np > 49152 && sums <= sm_count(); }
+
 }  // namespace
 
 void launch_area_total(const float4* patch_s, int64_t np, float* out, cudaStream_t stream) {
-    k_area_total<<<kSumBlocks, kSumThreads, 0, stream>>>(patch_s, (int)np, out);
+    if (split_sums(np, 1)) k_area_total_split<<<kSumBlocks, kSumChains / kSumBlocks, 0, stream>>>(patch_s, (int)np, out);
+    else k_area_total<<<1, kSumChains, 0, stream>>>(patch_s, (int)np, out);
 }
 
 namespace {
@@ -928,8 +962,11 @@ int fluence(const uvc_scene* sc, const float* A, int64_t nc, int64_t lda, const 
 
 int coverage(const uvc_scene* sc, const float* mu, int32_t nvec, float mu_min, float* cov_area, float* cov_count,
              cudaStream_t stream) {
-    k_coverage<<<nvec * kSumBlocks, kSumThreads, 0, stream>>>(mu, (int)sc->np, mu_min, sc->patch_s, sc->area_total, cov_area,
-                                          cov_count);
+    if (split_sums(sc->np, nvec))
+        k_coverage_split<<<nvec * kSumBlocks, kSumChains / kSumBlocks, 0, stream>>>(mu, (int)sc->np, mu_min, sc->patch_s,
+                                                                                   sc->area_total, cov_area, cov_count);
+    else
+        k_coverage<<<nvec, kSumChains, 0, stream>>>(mu, (int)sc->np, mu_min, sc->patch_s, sc->area_total, cov_area, cov_count);
     return status_from_cuda(cudaGetLastError());
 }
 
