@@ -12,13 +12,75 @@ namespace uvc {
 namespace {
 
 constexpr int kBins = 64;
-// Probe-column kernels: a block covers 8 columns x 128 row slices; thread
-// (slice, column) scans rows slice, slice + 128, ... (one 32-byte sector across
-// the 8 columns), and the slices are combined in shared memory.  The columns
-// are a probe's, a few hundred, so 32 columns x 8 slices left a dozen blocks
-// walking hundreds of rows one after the other (511 x 2,000: maxima 22 us,
-// marks 39 us, losses 127 us; now 6, 16 and 8 us).
-constexpr int kColW = 8, kColSlices = 128;
+// Probe-column kernels (k_col_max, k_mark_best, k_probe_lost): a block covers W
+// columns x SL row slices, thread (slice, column) scans rows slice, slice + SL,
+// ..., and the slices are combined by shuffles and in shared memory.  The shape
+// follows the number of columns: up to a block of 8 per SM (a probe's few hundred)
+// 128 slices keep the chain of rows short, up to eight such blocks 32 do, and wide
+// matrices read 128 bytes a row.  Marks of 511 x 2,000, 5,000 x 2,000 and 60,000 x
+// 2,000 (columns x rows), whole calls in us: 32 columns x 8 slices 42 / 43 / 117, 8
+// x 128 for all 39 / 60 / 389, by this rule 37 / 37 / 120.
+template <int W, int SL>
+struct Columns {
+    static constexpr int kW = W, kSlices = SL, kThreads = W * SL, kWarps = W * SL / 32;
+    static_assert(W <= 32 && 32 % W == 0 && W * SL <= 1024, "columns of a block");
+    __device__ static int column() { return (int)threadIdx.x % W; }
+    __device__ static int slice() { return (int)threadIdx.x / W; }
+    __device__ static int j() { return (int)blockIdx.x * W + column(); }
+    // f(row, A[row][j]) for this slice's rows in order, kAhead loads at a time (rows
+    // past the end give 0); ends after a batch of which f returned true for one.
+    static constexpr int kAhead = W == 32 ? 4 : 8;
+    template <class F>
+    __device__ static void rows_until(const float* __restrict__ A, int nc, int64_t lda, int j, F f) {
+        const float* p = A + (int64_t)slice() * lda + j;
+        const int64_t step = (int64_t)SL * lda;
+        bool done = false;
+        for (int64_t i = slice(); i < nc && !done; i += kAhead * SL, p += kAhead * step) {
+            float v[kAhead];
+            const bool whole = i + (kAhead - 1) * SL < nc;
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) v[u] = whole || i + u * SL < nc ? __ldg(p + u * step) : 0.f;
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) done |= f((int)i + u * SL, v[u]);
+        }
+    }
+    // All rows.  Wide matrices fill the chip with rows in flight as they are: a plain
+    // loop (marks of 60,000 x 2,000 in 120 us, by batches of 8 152, of 4 136).
+    template <class F>
+    __device__ static void rows(const float* __restrict__ A, int nc, int64_t lda, int j, F f) {
+        if constexpr (W == 32)
+            for (int i = slice(); i < nc; i += SL) f(i, A[(int64_t)i * lda + j]);
+        else
+            rows_until(A, nc, lda, j, [&](int i, float v) { f(i, v); return false; });
+    }
+    // v of this column's slices put together by `op`, in its slice-0 thread
+    template <class T, class Op>
+    __device__ static T combine(T v, T (*part)[W], Op op) {
+        for (int o = W; o < 32; o <<= 1) {
+            T other = v;
+            constexpr int kWords = sizeof(T) / 4;
+            int* w = reinterpret_cast<int*>(&other);
+#pragma unroll
+            for (int q = 0; q < kWords; ++q) w[q] = __shfl_down_sync(0xffffffffu, w[q], o);
+            v = op(v, other);
+        }
+        const int warp = (int)threadIdx.x >> 5;
+        if (((int)threadIdx.x & 31) < W) part[warp][column()] = v;
+        __syncthreads();
+        if (slice() == 0)
+            for (int q = 1; q < kWarps; ++q) v = op(v, part[q][column()]);
+        return v;
+    }
+};
+// f(shape) with the shape for np columns.
+template <class F>
+void with_columns(int64_t np, F f) {
+    const int64_t sms = sm_count();
+    if (np <= 8 * sms) f(Columns<8, 128>());
+    else if (np <= 64 * sms) f(Columns<8, 32>());
+    else f(Columns<32, 8>());
+}
+
 constexpr int kHistThreads = 256;
 
 struct Edges {
@@ -345,33 +407,26 @@ __global__ void __launch_bounds__(kSelectThreads) k_select_top(const float* __re
 }
 
 // Per probe patch j: its area if some candidate lights it (A[i][j] > 0) but
-// none of the selected ones does, else 0.
-__global__ void k_probe_lost(const float* __restrict__ A, int nc, int64_t lda, int np,
-                             const int32_t* __restrict__ idx, int k, const float* __restrict__ area,
-                             float* __restrict__ lost) {
-    __shared__ unsigned char pf[kColSlices][kColW], pr[kColSlices][kColW];
-    const int cx = threadIdx.x % kColW, sl = threadIdx.x / kColW;
-    const int j = blockIdx.x * kColW + cx;
+// none of the selected ones does, else 0.  Four rows at a time until one is lit.
+template <class C>
+__global__ void __launch_bounds__(C::kThreads) k_probe_lost(const float* __restrict__ A, int nc, int64_t lda, int np,
+                                                            const int32_t* __restrict__ idx, int k,
+                                                            const float* __restrict__ area, float* __restrict__ lost) {
+    __shared__ int part[C::kWarps][C::kW];
+    const int j = C::j(), sl = C::slice();
     bool full = false, red = false;
     if (j < np) {
-#pragma unroll 4
-        for (int i = sl; i < nc; i += kColSlices) full |= A[(int64_t)i * lda + j] > 0.f;
-#pragma unroll 4
-        for (int r = sl; r < k; r += kColSlices) {
-            const int i = idx[r];
-            if (i >= 0 && i < nc) red |= A[(int64_t)i * lda + j] > 0.f;   // rows out of range are ignored
+        C::rows_until(A, nc, lda, j, [&](int, float v) { return full |= v > 0.f; });
+        for (int r = sl; r < k && !red; r += 4 * C::kSlices) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = r + u * C::kSlices < k ? idx[r + u * C::kSlices] : -1;
+                if (i >= 0 && i < nc) red |= A[(int64_t)i * lda + j] > 0.f;   // rows out of range are ignored
+            }
         }
     }
-    pf[sl][cx] = full;
-    pr[sl][cx] = red;
-    __syncthreads();
-    if (sl == 0 && j < np) {
-        for (int q = 1; q < kColSlices; ++q) {
-            full |= pf[q][cx];
-            red |= pr[q][cx];
-        }
-        lost[j] = (full && !red) ? area[j] : 0.f;
-    }
+    const int m = C::combine((int)full | (int)red << 1, part, [](int x, int y) { return x | y; });
+    if (sl == 0 && j < np) lost[j] = m == 1 ? area[j] : 0.f;
 }
 
 // out = sum(lost) / sum(area), compensated sums in a fixed order (one block).
@@ -408,20 +463,15 @@ constexpr int kHardBins = 8, kEffBins = 6, kProbeFeat = kHardBins * kEffBins;
 constexpr int kProbeWarps = 4;
 
 // E*_j = max_i A[i][j].
-__global__ void k_col_max(const float* __restrict__ A, int nc, int64_t lda, int np, float* __restrict__ emax) {
-    __shared__ float part[kColSlices][kColW];
-    const int cx = threadIdx.x % kColW, sl = threadIdx.x / kColW;
-    const int j = blockIdx.x * kColW + cx;
+template <class C>
+__global__ void __launch_bounds__(C::kThreads) k_col_max(const float* __restrict__ A, int nc, int64_t lda, int np,
+                                                         float* __restrict__ emax) {
+    __shared__ float part[C::kWarps][C::kW];
+    const int j = C::j();
     float m = 0.f;
-    if (j < np)
-#pragma unroll 4
-        for (int i = sl; i < nc; i += kColSlices) m = fmaxf(m, A[(int64_t)i * lda + j]);
-    part[sl][cx] = m;
-    __syncthreads();
-    if (sl == 0 && j < np) {
-        for (int q = 1; q < kColSlices; ++q) m = fmaxf(m, part[q][cx]);
-        emax[j] = m;
-    }
+    if (j < np) C::rows(A, nc, lda, j, [&](int, float v) { m = fmaxf(m, v); });
+    m = C::combine(m, part, [](float x, float y) { return fmaxf(x, y); });
+    if (C::slice() == 0 && j < np) emax[j] = m;
 }
 
 // Lit-area-weighted mean of E* (compensated sums, fixed order, one block),
@@ -508,43 +558,38 @@ __global__ void __launch_bounds__(kProbeWarps * 32) k_probe_feat(const float* __
 // index among equal maxima); with rare > 0, also every candidate that lights
 // a patch lit by at most `rare` candidates.  Several patches may write the
 // same candidate with the same value.
-__global__ void k_mark_best(const float* __restrict__ A, int nc, int64_t lda, int np, float* __restrict__ score,
-                            float value, int rare) {
-    __shared__ float pv[kColSlices][kColW];
-    __shared__ int pi[kColSlices][kColW], pn[kColSlices][kColW];
-    const int cx = threadIdx.x % kColW, sl = threadIdx.x / kColW;
-    const int j = blockIdx.x * kColW + cx;
-    float m = 0.f;
-    int best = -1, lit = 0;
+struct Best {
+    float v;
+    int i, lit;   // row of the maximum (-1: none above 0), rows above 0
+};
+template <class C>
+__global__ void __launch_bounds__(C::kThreads) k_mark_best(const float* __restrict__ A, int nc, int64_t lda, int np,
+                                                           float* __restrict__ score, float value, int rare) {
+    __shared__ Best part[C::kWarps][C::kW];
+    __shared__ int lit[C::kW];
+    const int j = C::j(), sl = C::slice();
+    Best b{0.f, -1, 0};
     if (j < np)
-#pragma unroll 4
-        for (int i = sl; i < nc; i += kColSlices) {
-            const float v = A[(int64_t)i * lda + j];
-            lit += v > 0.f;
-            if (v > m) {        // rows ascend within a slice: the first maximum is kept
-                m = v;
-                best = i;
+        C::rows(A, nc, lda, j, [&](int i, float v) {
+            b.lit += v > 0.f;
+            if (v > b.v) {        // rows ascend within a slice: the first maximum is kept
+                b.v = v;
+                b.i = i;
             }
-        }
-    pv[sl][cx] = m;
-    pi[sl][cx] = best;
-    pn[sl][cx] = lit;
-    __syncthreads();
-    int total = 0;
-    for (int q = 0; q < kColSlices; ++q) total += pn[q][cx];
-    if (sl == 0 && j < np) {
-        for (int q = 1; q < kColSlices; ++q) {
-            const float v = pv[q][cx];
-            const int b = pi[q][cx];
-            if (b >= 0 && (v > m || (v == m && (best < 0 || b < best)))) {
-                m = v;
-                best = b;
-            }
-        }
-        if (best >= 0) score[best] = value;
+        });
+    b = C::combine(b, part, [](Best x, Best y) {
+        const bool other = y.i >= 0 && (y.v > x.v || (y.v == x.v && (x.i < 0 || y.i < x.i)));
+        return Best{other ? y.v : x.v, other ? y.i : x.i, x.lit + y.lit};
+    });
+    if (sl == 0) {
+        lit[C::column()] = b.lit;
+        if (j < np && b.i >= 0) score[b.i] = value;
     }
+    if (rare <= 0) return;
+    __syncthreads();
+    const int total = lit[C::column()];
     if (j < np && total > 0 && total <= rare)
-        for (int i = sl; i < nc; i += kColSlices)
+        for (int i = sl; i < nc; i += C::kSlices)
             if (A[(int64_t)i * lda + j] > 0.f) score[i] = value;
 }
 
@@ -578,9 +623,12 @@ int group_boost(float* score, int64_t n, int group, float bonus, cudaStream_t st
 
 int mark_best(const float* A, int64_t nc, int64_t lda, int64_t np, float* score, float value, int rare,
               cudaStream_t stream) {
-    if (np > 0 && nc > 0)
-        k_mark_best<<<(int)((np + kColW - 1) / kColW), kColW * kColSlices, 0, stream>>>(A, (int)nc, lda, (int)np,
-                                                                                      score, value, rare);
+    if (np > 0 && nc > 0) {
+        with_columns(np, [&](auto shape) {
+            using C = decltype(shape);
+            k_mark_best<C><<<(int)((np + C::kW - 1) / C::kW), C::kThreads, 0, stream>>>(A, (int)nc, lda, (int)np, score, value, rare);
+        });
+    }
     return status_from_cuda(cudaGetLastError());
 }
 
@@ -590,8 +638,12 @@ int probe_features(const float* A, int64_t nc, int64_t lda, int64_t np, const fl
     float* emax = work;
     float* stats = work + np;
     signed char* hb = reinterpret_cast<signed char*>(work + np + 4);
-    if (np > 0)
-        k_col_max<<<(int)((np + kColW - 1) / kColW), kColW * kColSlices, 0, stream>>>(A, (int)nc, lda, (int)np, emax);
+    if (np > 0) {
+        with_columns(np, [&](auto shape) {
+            using C = decltype(shape);
+            k_col_max<C><<<(int)((np + C::kW - 1) / C::kW), C::kThreads, 0, stream>>>(A, (int)nc, lda, (int)np, emax);
+        });
+    }
     k_probe_bins<<<1, 256, 0, stream>>>(emax, area, (int)np, stats, hb);
     k_probe_feat<<<(int)((nc + kProbeWarps - 1) / kProbeWarps), kProbeWarps * 32, 0, stream>>>(
         A, (int)nc, lda, (int)np, emax, hb, area, stats, feat, ldf);
@@ -601,8 +653,10 @@ int probe_features(const float* A, int64_t nc, int64_t lda, int64_t np, const fl
 int probe_lost(const float* A, int64_t nc, int64_t lda, int64_t np, const int32_t* idx, int64_t k,
                const float* area, float* lost, float* out, cudaStream_t stream) {
     if (np > 0) {
-        k_probe_lost<<<(int)((np + kColW - 1) / kColW), kColW * kColSlices, 0, stream>>>(A, (int)nc, lda, (int)np, idx,
-                                                                                       (int)k, area, lost);
+        with_columns(np, [&](auto shape) {
+            using C = decltype(shape);
+            k_probe_lost<C><<<(int)((np + C::kW - 1) / C::kW), C::kThreads, 0, stream>>>(A, (int)nc, lda, (int)np, idx, (int)k, area, lost);
+        });
     }
     k_probe_total<<<1, 256, 0, stream>>>(lost, area, (int)np, out);
     return status_from_cuda(cudaGetLastError());
