@@ -653,7 +653,8 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
 
 // The lane's patch (its flag bit: plates.cu, k_plate_patches).  A patch on an
 // axis plane that has a clearance has no triangle of that plane but its own
-// within 2^-14 of the scene's diagonal (build_bvh.cu: k_clearance).
+// within 2^-14 of the scene's diagonal, nor within the clearance if that is less:
+// the search for it looks at nothing farther away (build_bvh.cu: k_clearance).
 __device__ __forceinline__ PlateLane plate_lane(const SceneView& S, int jb, int lane, const PatchLane& P) {
     PlateLane pl;
     pl.flagged = (__ldg(reinterpret_cast<const uint32_t*>(S.plates + 2 * kMaxPlates) + jb) >> lane) & 1u;
@@ -662,7 +663,7 @@ __device__ __forceinline__ PlateLane plate_lane(const SceneView& S, int jb, int 
                       (z && P.n.x == 0.f && P.n.y == 0.f);
     pl.own_axis = unit && P.n.w > 0.f ? (x ? 0 : (y ? 1 : 2)) : -1;
     pl.own = x ? P.s.x : (y ? P.s.y : P.s.z);
-    pl.gap = S.cut_eps * 6.f;   // 1e5 2^-14 = 6.1
+    pl.gap = fminf(S.cut_eps * 6.f, P.n.w);   // 1e5 2^-14 = 6.1
     pl.plate = -1;
     return pl;
 }
