@@ -214,8 +214,24 @@ __global__ void __launch_bounds__(kThreads, PLATES ? kCallMinBlocks : UVC_IRR_MI
         // the check points' gaps, where plates are in use and the patch and its
         // excluded triangles lie in one axis plane
         float gap[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        unsigned off = 0u;   // bit q: check point q lies out of the plane of an excluded triangle's plate
         PlateLane plc = pl;
         plc.plate = -1;
+        if (PLATES && S.nplate != 0 && L.plates)
+#pragma unroll 1
+            for (int t = 0; t < 2; ++t) {
+                const int id = t ? P.ex.y : P.ex.x;
+                const int plate = id >= 0 ? __ldg(&tri_place[id]).y : -1;
+                if (plate < 0) continue;
+                const float4 lo = __ldg(&S.plates[2 * plate]);
+                const int ax = __float_as_int(lo.w);
+#pragma unroll 1
+                for (int q = 0; q < 6; ++q) {
+                    if (!((tmask >> (q / 3)) & 1)) continue;
+                    const float3 v = pulled(vertex(g, q), P.s);
+                    if (pick(v.x, v.y, v.z, ax) != pick(lo.x, lo.y, lo.z, ax)) off |= 1u << q;
+                }
+            }
         if (PLATES && S.nplate != 0 && L.plates && pl.own_axis >= 0) {
             float2 T[2][3];
             bool in[2] = {false, false};
@@ -274,6 +290,7 @@ __global__ void __launch_bounds__(kThreads, PLATES ? kCallMinBlocks : UVC_IRR_MI
 #pragma unroll
                         for (int k = 0; k < 6; ++k) plq.gap = q == k ? gap[k] : plq.gap;   // no indexed registers
                         if (!(plq.gap > 0.f)) plq.own_axis = -1;
+                        plq.flagged = plq.flagged || ((off >> q) & 1u);
                     }
                     uint32_t fq;
                     const uint32_t oc = wedge_search<false, PLATES, PLATES, PLATES>(S, L, cx, cy, cz, szq, gxq, gyq, want_q, lq, dq, P.ex, plq, lane, stack, ws, cache, fq, nullptr);
