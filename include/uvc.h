@@ -358,7 +358,8 @@ int uvc_coverage(const uvc_scene* scene, const float* mu, int32_t nvec, float mu
  * e.g. rooms of uneven size crossed with lamp designs (the robot-design
  * comparison of Sec. V-C) - computed by one persistent launch whose warps walk
  * the tasks of all jobs round-robin, so the launch ends evenly whatever the
- * job sizes.  Each job writes its own A (and optional visibility words)
+ * job sizes (two where some jobs' scenes have plates and others' do not, see
+ * uvc_set_wedge_traversal).  Each job writes its own A (and optional visibility words)
  * exactly as uvc_irradiance_matrix would (bit-identical results).
  *
  *   uvc_job.scene, cand, nc, A, lda, vis  as in uvc_irradiance_matrix

@@ -4,8 +4,8 @@
 // The tasks of all jobs (one task = 32 patches x a chunk of candidates, as in
 // k_irradiance) form one flat index space, job after job.  A persistent grid
 // walks it round-robin, so every warp sees a mix of big and small jobs and
-// the launch ends evenly whatever the job sizes.  The job table lives in
-// device memory the caller provides; uvc_batch_launch reads no host data and
+// the launch ends evenly whatever the job sizes.  (Jobs with plates and jobs
+// without get a launch each.)  The job table lives in device memory the caller provides; uvc_batch_launch reads no host data and
 // allocates nothing, so it can be captured in a CUDA graph and replayed.
 // The autotuner times the tunable launch parameters (candidates per task,
 // resident blocks per SM) on a sample of the tasks and keeps the fastest.
@@ -51,7 +51,10 @@ static_assert(sizeof(LampPack) + 64 <= 32764, "kernel parameters");
 // arrays, sized for the batch's largest such lamp (wedge_k).  MODE: 0 = no
 // lamp of the batch takes the wedge path, 1 = all do, 2 = mixed (chosen per
 // job; both paths inlined).  PACK: the lamps and jobs come from `pack`.  PLATES:
-// some job's scene has plates.
+// jobs whose scenes have plates.  They come first in the table and the others get
+// a launch of their own: two blocks per SM with a called search, which plates want,
+// cost the others 5 % and more in one launch (one small room of plates among three
+// turned ones 30.8 ms, in two launches 29.2; three of four with plates 17.3 and 15.6).
 template <int MODE, bool PACK, bool PLATES>
 __global__ void __launch_bounds__(kThreads, PLATES ? kCallMinBlocks : UVC_IRR_MIN_BLOCKS)
     k_irradiance_batch(const JobDev* __restrict__ jobs, int njobs, const LampDev* __restrict__ lamps,
@@ -110,14 +113,13 @@ struct uvc_batch {
     int device = 0;
     int njobs = 0, nlamps = 0;
     std::vector<uvc::JobDev> host_jobs;   // task_begin filled per config
-    std::vector<int64_t> pairs;           // nc * np per job
     std::vector<uvc::LampDev> host_lamps;
     uvc::JobDev* dev_jobs = nullptr;      // in the caller's workspace
     uvc::LampDev* dev_lamps = nullptr;
     int stack_cap = 1;
     int wedge_k = 0;                      // largest K among the lamps with the wedge path
     int mode = 0;                         // kernel variant: 0 no wedge lamp, 1 all wedge, 2 mixed
-    bool plates = false;                  // some job decides segments at plates
+    int plate_jobs = 0;                   // the first jobs: they decide segments at plates
     int64_t total_pairs = 0;
     uvc::LampPack pack{};                 // the lamps and jobs again, for the kernel parameters (small batches)
     int uploaded_cpt = 0;                 // cand_per_task of the uploaded table
@@ -149,10 +151,10 @@ int upload(uvc_batch* b, int cpt, cudaStream_t stream, int64_t* total_tasks) {
     return UVC_OK;
 }
 
-int launch_range(const uvc_batch* b, int cpt, int blocks_per_sm, int64_t lo, int64_t hi, cudaStream_t stream) {
+int launch_part(const uvc_batch* b, bool plates, int cpt, int blocks_per_sm, int64_t lo, int64_t hi, cudaStream_t stream) {
     if (hi <= lo) return UVC_OK;
     const bool pack = b->nlamps <= kParamLamps && b->njobs <= kParamJobs;
-    BatchKernel k = kernel_for(b->mode, pack, b->plates);
+    BatchKernel k = kernel_for(b->mode, pack, plates);
     const size_t smem = stack_smem_bytes(b->stack_cap) + wedge_smem_bytes(b->wedge_k);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -169,6 +171,13 @@ int launch_range(const uvc_batch* b, int cpt, int blocks_per_sm, int64_t lo, int
     k<<<(int)grid, kThreads, smem, stream>>>(b->dev_jobs, b->njobs, b->dev_lamps, b->pack, cpt, lo, hi, b->stack_cap,
                                              b->wedge_k);
     return status_from_cuda(cudaGetLastError());
+}
+
+// The tasks [lo, hi) of the configuration that fill_task_begin has last laid out.
+int launch_range(const uvc_batch* b, int cpt, int blocks_per_sm, int64_t lo, int64_t hi, cudaStream_t stream) {
+    const int64_t line = b->plate_jobs < b->njobs ? b->host_jobs[b->plate_jobs].task_begin : hi;
+    const int rc = launch_part(b, true, cpt, blocks_per_sm, lo, std::min(hi, line), stream);
+    return rc != UVC_OK ? rc : launch_part(b, false, cpt, blocks_per_sm, std::max(lo, line), hi, stream);
 }
 
 // size bucket of a batch for the tuning cache: log2 of its pairs and of its mean sources
@@ -225,7 +234,6 @@ int uvc_batch_create(const uvc_job* jobs, int32_t njobs, const uvc_lamp* lamps, 
     for (const auto& D : b->host_lamps) nwedge += D.wedge ? 1 : 0;
     b->mode = nwedge == 0 ? 0 : (nwedge == nlamps ? 1 : 2);
     b->host_jobs.resize(njobs);
-    b->pairs.resize(njobs);
     int maxcap = 1;
     for (int q = 0; q < njobs; ++q) {
         const uvc_job& J = jobs[q];
@@ -237,7 +245,6 @@ int uvc_batch_create(const uvc_job* jobs, int32_t njobs, const uvc_lamp* lamps, 
         }
         uvc::JobDev& D = b->host_jobs[q];
         D.S = uvc::view_of(J.scene);
-        b->plates |= D.S.nplate != 0 && b->host_lamps[J.lamp].plates;
         D.cand = J.cand;
         D.A = J.A;
         D.vis = J.vis;
@@ -246,11 +253,14 @@ int uvc_batch_create(const uvc_job* jobs, int32_t njobs, const uvc_lamp* lamps, 
         D.lamp = J.lamp;
         D.njb = (int)((J.scene->np + 31) / 32);
         if (J.nc == 0) D.njb = 0;   // nothing to do for this job
-        b->pairs[q] = J.nc * J.scene->np;
-        b->total_pairs += b->pairs[q];
+        b->total_pairs += J.nc * J.scene->np;
         maxcap = std::max(maxcap, D.S.stack_cap);
     }
     b->stack_cap = maxcap;
+    const auto others = std::stable_partition(b->host_jobs.begin(), b->host_jobs.end(), [&](const uvc::JobDev& D) {
+        return D.S.nplate != 0 && b->host_lamps[D.lamp].plates;
+    });
+    b->plate_jobs = (int)(others - b->host_jobs.begin());
     char* ws = static_cast<char*>(workspace);
     b->dev_jobs = reinterpret_cast<uvc::JobDev*>(ws);
     b->dev_lamps = reinterpret_cast<uvc::LampDev*>(ws + ((sizeof(uvc::JobDev) * (size_t)njobs + 255) & ~size_t(255)));

@@ -679,7 +679,7 @@ def irradiance_candidates_per_task() -> int:
 
 
 class Batch:
-    """Many irradiance matrices in one persistent launch (uvc_batch_*).
+    """Many irradiance matrices in one persistent launch, or two (uvc_batch_*).
 
     jobs: list of (scene, cand (nc,3) CUDA tensor, lamp index, A (nc, lda) CUDA
     tensor, vis CUDA int32 tensor or None); lamps: list of Lamp.  The caller
