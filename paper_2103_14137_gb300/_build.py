@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libuvc.so")
 SOURCES = ["build_bvh.cu", "plates.cu", "irradiance.cu", "batch.cu", "fluence.cu", "solid_angle.cu", "raster.cu", "features.cu", "mlp.cu", "probe.cu", "api.cu"]
-HEADERS = ["uvc_internal.cuh", "traverse.cuh", "tcgen05.cuh", "collapse_plan.h"]
+HEADERS = ["uvc_internal.cuh", "traverse.cuh", "tcgen05.cuh", "collapse_plan.h", "raster_box.h"]
 INCLUDE = os.path.join(HERE, "..", "include")
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]

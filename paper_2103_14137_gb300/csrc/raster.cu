@@ -36,6 +36,7 @@
 #include <mutex>
 #include <vector>
 
+#include "raster_box.h"
 #include "uvc_internal.cuh"
 
 namespace uvc {
@@ -196,18 +197,10 @@ __global__ void __launch_bounds__(256) k_rs_setup(RasterBatch B, float near_eps)
             if (umax >= -1.f && umin <= 1.f && vmax >= -1.f && vmin <= 1.f) {
                 umin = fmaxf(umin, -1.f); umax = fminf(umax, 1.f);
                 vmin = fmaxf(vmin, -1.f); vmax = fminf(vmax, 1.f);
-                const float h = 0.5f * B.R;
-                // pixel centres (2p + 1) / R - 1 inside [min, max], widened: the
-                // projection and the ray test move a vertex by less than 2^-20 of
-                // its distance over its depth, so 1/32 of a pixel covers up to
-                // R = 4096 where no depth is below 1/16 of the distances; other
-                // triangles (next to the source's own plane) get two pixels
-                const float e = wlo * 16.f >= reach ? 0.03125f : 2.f;
-                const int x0 = max(0, (int)ceilf((umin + 1.f) * h - 0.5f - e));
-                const int x1 = min(B.R - 1, (int)floorf((umax + 1.f) * h - 0.5f + e));
-                const int y0 = max(0, (int)ceilf((vmin + 1.f) * h - 0.5f - e));
-                const int y1 = min(B.R - 1, (int)floorf((vmax + 1.f) * h - 0.5f + e));
-                if (x1 >= x0 && y1 >= y0) bx = make_uint2((unsigned)x0 | ((unsigned)x1 << 16), (unsigned)y0 | ((unsigned)y1 << 16));
+                const bool deep = wlo * 16.f >= reach;
+                const PixelRange x = pixel_range(umin, umax, B.R, deep), y = pixel_range(vmin, vmax, B.R, deep);
+                if (x.last >= x.first && y.last >= y.first)
+                    bx = make_uint2((unsigned)x.first | ((unsigned)x.last << 16), (unsigned)y.first | ((unsigned)y.last << 16));
             }
         }
         const int face = c * 6 + f;
