@@ -5,8 +5,9 @@
 // k_irradiance) form one flat index space, job after job.  A persistent grid
 // walks it round-robin, so every warp sees a mix of big and small jobs and
 // the launch ends evenly whatever the job sizes.  (Jobs with plates and jobs
-// without get a launch each.)  The job table lives in device memory the caller provides; uvc_batch_launch reads no host data and
-// allocates nothing, so it can be captured in a CUDA graph and replayed.
+// without get a launch each.)  The job table lives in device memory the caller
+// provides; uvc_batch_launch reads no host data and allocates nothing, so it can
+// be captured in a CUDA graph and replayed.
 // The autotuner times the tunable launch parameters (candidates per task,
 // resident blocks per SM) on a sample of the tasks and keeps the fastest.
 #include <algorithm>
@@ -254,7 +255,7 @@ int uvc_batch_create(const uvc_job* jobs, int32_t njobs, const uvc_lamp* lamps, 
         D.njb = (int)((J.scene->np + 31) / 32);
         if (J.nc == 0) D.njb = 0;   // nothing to do for this job
         b->total_pairs += J.nc * J.scene->np;
-        maxcap = std::max(maxcap, D.S.stack_cap);
+        maxcap = std::max<int>(maxcap, D.S.stack_cap);
     }
     b->stack_cap = maxcap;
     const auto others = std::stable_partition(b->host_jobs.begin(), b->host_jobs.end(), [&](const uvc::JobDev& D) {

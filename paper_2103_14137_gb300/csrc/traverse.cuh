@@ -51,13 +51,16 @@ struct SceneView {
     const int2* __restrict__ pe;
     const float4* __restrict__ plates;   // [kMaxPlates][2], then the patch flag words
     int nt, np;
-    int nplate;      // plates in use; kLooseBit set when triangles lie outside them
-    int stack_cap, visit_cap;
+    uint16_t nplate;      // plates in use; kLooseBit set when triangles lie outside them
+    uint16_t stack_cap;
+    int visit_cap;
     float cut_eps;   // absolute slack (metres) subtracted from a patch's clearance
+    float plate_eps;   // widening of a plate's box
     int* status;
 };
 
-constexpr int kLooseBit = 1 << 30;
+constexpr int kLooseBit = 1 << 15;
+static_assert(kMaxPlates < kLooseBit, "plates and their flag in 16 bits");
 // Root reference: node 0, or the only triangle.
 __device__ __forceinline__ int root_of(const SceneView& S) { return S.nt == 1 ? ~0 : 0; }
 
@@ -73,12 +76,17 @@ SceneView view_of(const uvc_scene* sc) {
     // a scene with lowered limits searches the hierarchy for everything
     const bool plates = sc->nplate > 0 && sc->limit_stack <= 0 && sc->limit_visits <= 0;
     v.plates = sc->plates;
-    v.nplate = plates ? (sc->nplate | (sc->nloose > 0 ? kLooseBit : 0)) : 0;
-    v.stack_cap = 3 * (sc->depth4 + 1) + 1;   // at most 3 pushes per four-wide level
+    v.nplate = (uint16_t)(plates ? (sc->nplate | (sc->nloose > 0 ? kLooseBit : 0)) : 0);
+    // at most 3 pushes per four-wide level; a stack of 2^16 would not fit a block's
+    // shared memory, its launch is refused
+    v.stack_cap = (uint16_t)std::min(3 * ((int64_t)sc->depth4 + 1) + 1, (int64_t)65535);
     v.visit_cap = (int)sc->nt + 64;
-    if (sc->limit_stack > 0 && sc->limit_stack < v.stack_cap) v.stack_cap = sc->limit_stack;
+    if (sc->limit_stack > 0 && sc->limit_stack < v.stack_cap) v.stack_cap = (uint16_t)sc->limit_stack;
     if (sc->limit_visits > 0 && sc->limit_visits < v.visit_cap) v.visit_cap = sc->limit_visits;
     v.cut_eps = 1e-5f * sc->diameter;
+    // the box tests round absolute coordinates, by up to 2^-22 of them in all: in a
+    // scene far from the origin that is more than cut_eps
+    v.plate_eps = v.cut_eps + 4.76837158203125e-07f * sc->coord_bound;   // 2^-21
     v.status = sc->status;
     return v;
 }
@@ -438,7 +446,8 @@ __device__ __forceinline__ PatchLane load_patch(const SceneView& S, int j) {
 // per lane, against the packet's shaft: the hull's box, the two vertical
 // planes through the column that hold all points, and the two slanted planes
 // below and above.  The rectangles are widened by twice the box tests' own
-// widening, so the shaft misses no box test that would hit.
+// widening, so the shaft misses no box test that would hit.  The box tests here
+// are widened by more than the search's (SceneView::plate_eps).
 // Measured on a ward (49,066 triangles in 66 plates, 98,132 x 2,000 pairs,
 // K = 8): matrix 55.4 -> 10.5 ms, 7.45 with the set-up by surface and the lamp's
 // ends tested first (ENDS: set-up 2.3 ms, shaft 0.7, cull 1.2, 1.2 rectangles hit
@@ -516,7 +525,7 @@ __device__ __forceinline__ uint32_t plates_decide(const SceneView& S, Z zsrc, in
                                                   const Slabs& sl, const PlateLane& pl, int lane, uint32_t& want) {
     const float kBig = 3.0e38f, kWide = 4.76837158203125e-07f;   // 2^-21: the rounding of a rectangle's middle and half width
     const bool a0 = want != 0u;
-    const float delta = S.cut_eps, diag = S.cut_eps * 1e5f;
+    const float delta = S.plate_eps, diag = S.cut_eps * 1e5f;
     // far outside the scene (or infinite, or NaN) the widening no longer covers the rounding of the shaft
     if (__any_sync(kFull, a0 && !(dmax < 32.f * diag))) return want;
     // the packet's shaft, relative to the column's foot in x and y
@@ -704,7 +713,7 @@ __device__ __forceinline__ float irradiance_entry(const SceneView& S, const floa
         const uint32_t before = want;
         if (plates && __any_sync(kFull, want))
             open = plates_decide<false>(S, [&](int) { return oz; }, 1, ox, oy, s4.z, -hx, -hy, oz, oz,
-                                 tend, d, slabs_of(ox, oy, -hx, -hy, S.cut_eps), pl, lane, want);
+                                 tend, d, slabs_of(ox, oy, -hx, -hy, S.plate_eps), pl, lane, want);
         for (int whole = plates && (S.nplate & kLooseBit) ? 0 : 1; whole < 2; ++whole) {
             const uint32_t search = __ballot_sync(kFull, want && (whole ? open : !open));
             if (!search) continue;
@@ -1420,7 +1429,7 @@ __device__ __forceinline__ uint32_t wedge_search(const SceneView& S, const LampD
     if (S.nt == 0 || !__any_sync(kFull, want != 0u)) return 0u;
     const uint32_t before = want;
     const bool plates = PLATES && S.nplate != 0 && L.plates;
-    const Slabs sl = slabs_of(cx, cy, gx, gy, S.cut_eps);
+    const Slabs sl = slabs_of(cx, cy, gx, gy, plates ? S.plate_eps : S.cut_eps);
     uint32_t open = want;
     if (plates) {
         float zlo = __fadd_rn(cz, L.zmin), zhi = __fadd_rn(cz, L.zmax);
