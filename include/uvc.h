@@ -163,12 +163,15 @@ int uvc_set_fluence_tensor_cores(int32_t enable, int32_t* previous);
  * source by source with the same segment test; they can differ only where a
  * segment grazes a triangle lying in the patch's own plane.  Scenes of more
  * than 2^27 triangles are always searched source by source.
- * With 1, all lamps also decide segments at the scene's plates first (flat
+ * With 1, segments are also decided at the scene's plates first (flat
  * axis-parallel rectangles that the mesh tiles completely, found by
- * uvc_build_scene); with 0 the hierarchy is searched for everything.  The
+ * uvc_build_scene), by all lamps, but in uvc_irradiance_area_mean by vertical
+ * line lamps only; with 0 the hierarchy is searched for everything.  The
  * results are the same: a plate decides only segments that pass its borders
  * and its plane by more than the segment test's rounding, and the hierarchy
- * is searched for the rest.  Scenes with lowered limits do not use plates.
+ * is searched for the rest.  Scenes with lowered limits do not use plates, nor
+ * do scenes of more than 1,024 of them or with more than eight loose triangles
+ * for each triangle of the plates inside their bounds.
  * The setting is read when a call (or uvc_batch_create) converts its lamp.
  *   enable    0 or 1
  *   previous  HOST int32, may be NULL: receives the setting before the call
