@@ -42,7 +42,7 @@ __device__ __forceinline__ void kahan_add(float& sum, float& c, float x) {
 // The first form had one block per 128 columns and all candidates in 4 groups,
 // four rows ahead, one launch per 16 vectors: on a 697 x 9,273 matrix, 73 blocks
 // for 54 us a launch, each thread waiting for its next four rows.  With 37
-// vectors there, fluence and coverage together: 164 -> 70 us.
+// vectors there, fluence and coverage together: 164 -> 76 us.
 constexpr int kFlGroups = 4;                      // row groups per block
 constexpr int kFlGroupThreads = 64;              // threads per row group
 constexpr int kFlCols = 2 * kFlGroupThreads;     // columns per block
@@ -259,10 +259,10 @@ __global__ void __launch_bounds__(256, 2) k_fluence_wide(const float* __restrict
 // loaded by cp.async.bulk.tensor (one 2-D tensor-map copy per tile, issued by
 // the group's first thread) and completed on an mbarrier per tile.  Up to
 // 4 groups x kTmaStages tiles = 128 KB per SM are in flight without
-// occupying a register, where k_fluence has 16 KB.  The grid is persistent
+// occupying a register, where k_fluence_wide has 16 KB.  The grid is persistent
 // (one block per SM, looping over the 128-column strips).  Needs rows that
 // start on 16-byte boundaries (lda a multiple of 4, A 16-byte aligned); other
-// layouts take k_fluence.  Every wait is bounded: a wait that runs out
+// layouts take k_fluence_wide.  Every wait is bounded: a wait that runs out
 // records UVC_E_TIMEOUT in the scene's status word and the block finishes
 // without further waiting (its results are then invalid).
 constexpr int kTmaRows = 16;                      // rows per tile
